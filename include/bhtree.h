@@ -56,7 +56,9 @@ typedef struct bh_config {
     int order;               /* 1 = monopole (the paper), 2 = monopole + quadrupole */
     int fp64_node_threshold; /* nodes holding >= this many particles combine moments in FP64 */
     int block_threads;       /* threads per block of the walk kernel: 64 or 128 */
-    int blocks_per_sm;       /* resident walk blocks per SM for the persistent grid (0 = auto) */
+    int blocks_per_sm;       /* resident walk blocks per SM for the persistent grid (0 = auto;
+                                a set with few groups then takes a block of warps per group,
+                                with the same bits) */
     int max_systems;         /* independent systems one bh_force_batched call may hold (>= 1) */
     int curve;               /* particle order (Sec. 5): BH_CURVE_MORTON (default) or
                                 BH_CURVE_HILBERT (Peano-Hilbert); the octree is the same,

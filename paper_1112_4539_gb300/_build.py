@@ -18,7 +18,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 # per-file extra flags: the walk's interaction loops flush denormals (positions
 # and softened distances are far from the denormal range)
-EXTRA = {"bh_walk.cu": ["-ftz=true"]}
+EXTRA = {"bh_walk.cu": ["-ftz=true"], "bh_walk_team.cu": ["-ftz=true"]}
 
 
 def sources():

@@ -378,7 +378,7 @@ int tree_force(bh_ctx* x, float eps, float* d_acc_pot, void* stream)
     bh::WalkLearned wl{x->mfeat, x->mlp, x->theta};
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, x->nd, x->cfg.order, x->cfg.group_size,
                              eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
-                             x->cfg.blocks_per_sm, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
+                             x->cfg.blocks_per_sm, (int)x->n, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     x->launches += bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
@@ -749,7 +749,7 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
                        x->cfg.curve, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, x->nd, x->cfg.order, x->cfg.group_size, eps,
-                             (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads, x->cfg.blocks_per_sm, s,
+                             (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     // init, batch sort, 4 tree, 5 groups, moments per level, 2 walk

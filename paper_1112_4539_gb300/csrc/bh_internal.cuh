@@ -363,7 +363,7 @@ struct WalkLearned {
 };
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl,
-                int sm_count, int block_threads, int blocks_per_sm, cudaStream_t s,
+                int sm_count, int block_threads, int blocks_per_sm, int n, cudaStream_t s,
                 const WalkLearned* learned = nullptr, int walk_variant = 0);
 // failure-path self-tests: one bounded wait that nothing satisfies
 void launch_selftest_ring(bh_dev_ctrl* c, cudaStream_t s);

@@ -1246,7 +1246,7 @@ static int bh_walk_dispatch(const WalkParams& P, int order, int G, int sm_count,
 
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl, int sm_count,
-                int block_threads, int blocks_per_sm, cudaStream_t s, const WalkLearned* learned, int walk_variant)
+                int block_threads, int blocks_per_sm, int n, cudaStream_t s, const WalkLearned* learned, int walk_variant)
 {
     bh_walk_reset_kernel<<<1, 1, 0, s>>>(ctrl);
     WalkParams P;
@@ -1265,6 +1265,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
     P.mlp = nullptr;
     P.theta_guard = 1.0f;
     P.wrec = nd.wrec;
+    P.sm_count = sm_count;
     if (learned) {
         P.mfeat = learned->mfeat;
         P.mlp = learned->mlp;
@@ -1287,6 +1288,11 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
             case 2: return bh_walk_ws_launch<2, 1>(P, sm_count, s);
             default: return bh_walk_ws_launch<3, 1>(P, sm_count, s);
         }
+    }
+    // few groups: a block of warps each (same bits), unless the caller sized the grid
+    if (blocks_per_sm == 0) {
+        const int rc = launch_walk_team(P, order, G, n, sm_count, s);
+        if (rc <= 0) return rc;
     }
     return bh_walk_dispatch<false>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
 }

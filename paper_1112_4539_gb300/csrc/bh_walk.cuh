@@ -1,4 +1,6 @@
-// bh_walk.cuh -- device code shared by the group-walk kernels: the shared-memory staging of sources, the tile arithmetic on packed source
+// bh_walk.cuh -- device code shared by the group-walk kernels (bh_walk.cu: one
+// warp per group, warp pairs, TMA staging; bh_walk_team.cu: a block per group):
+// the shared-memory staging of sources, the tile arithmetic on packed source
 // pairs, the layout of a group's targets on a warp, and bounded mbarrier waits.
 #pragma once
 
@@ -106,6 +108,7 @@ struct WalkParams {
     const bh_mlp_dev* mlp;   // network (global copy)
     float theta_guard;       // theta of the S_eff in use (the guard)
     const float4* wrec;      // walk records (TMA-staged walk)
+    int sm_count;
 };
 
 // Running totals of a lane's T targets with their Kahan compensations, the
@@ -550,5 +553,10 @@ __device__ __forceinline__ int bh_take_particles(int2* q, int& pos, int n, unsig
     pos += nfull;
     return min(total, 32);
 }
+
+// A block of warps per group (bh_walk_team.cu), for few enough groups of at most
+// kTeamMaxGroup targets: a BH_* code, or 1 when the set is not for it.
+constexpr int kTeamMaxGroup = 128;
+int launch_walk_team(const WalkParams& P, int order, int G, int n, int sm_count, cudaStream_t s);
 
 }  // namespace bh

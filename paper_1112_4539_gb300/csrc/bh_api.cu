@@ -396,7 +396,7 @@ int tree_force_particles(bh_ctx* x, float eps, int flags, float* d_acc_pot, void
     if (x->n == 0) return BH_OK;
     if (!d_acc_pot || !aligned16(d_acc_pot) || !is_device_ptr(d_acc_pot, x->device)) return BH_ERR_INVALID;
     DeviceGuard guard(x->device);
-    int rc = bh::launch_pwalk(x->pos_s, x->vals, x->nd, x->parent, x->next, x->cfg.order, (int)x->n,
+    int rc = bh::launch_pwalk(x->pos_s, x->vals, x->nd, x->parent, x->next, x->cfg.order, x->deep, (int)x->n,
                               (int)x->node_cap, eps, (flags & BH_PWALK_UNSOFTENED_CELLS) != 0, (float4*)d_acc_pot,
                               x->ctrl, x->sm_count, (cudaStream_t)stream, ind ? &x->soft : nullptr);
     if (rc) return rc;

@@ -383,7 +383,7 @@ struct bh_soft {
     float* hbar = nullptr;     // per node
 };
 int launch_pwalk(const float4* pos_s, const uint32_t* perm, const bh_nodes& nd, int32_t* parent, int32_t* next,
-                 int order, int n, int node_cap, float eps, bool unsoftened_cells, float4* out, bh_dev_ctrl* ctrl,
+                 int order, bool deep, int n, int node_cap, float eps, bool unsoftened_cells, float4* out, bh_dev_ctrl* ctrl,
                  int sm_count, cudaStream_t s, const bh_soft* soft = nullptr);
 void launch_softening(const float* eps, const uint32_t* perm, const float4* pos_s, const bh_nodes& nd, int n,
                       bool deep, const bh_soft& soft, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);

@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
         bool overflow = false;
         while (sp > 0) {
             // ---- pop the top 32 nodes (ranges of siblings)
-            int v;
-            const int npop = bh_pop_nodes(S.stack, sp, lt, v);
+            int v, row;
+            const int npop = bh_pop_nodes(S.stack, sp, lt, v, row);
             const bool has = lane < npop;
             v = has ? v : 0;
             __syncwarp();
@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
                     continue;
                 }
                 if (lq_pos >= lq_n) break;
-                int k;
-                const int nfill = bh_take_particles(S.leafq, lq_pos, lq_n, lt, k);
+                int k, row;
+                const int nfill = bh_take_particles(S.leafq, lq_pos, lq_n, lt, k, row);
                 if (lane < nfill) bh_put_point(S, (ring_head + ring_cnt + lane) & (kRing - 1), P.pos_s[k]);
                 ring_cnt += nfill;
                 __syncwarp();

@@ -500,8 +500,9 @@ __device__ __forceinline__ bool bh_mbar_wait(unsigned long long* b, unsigned int
 
 // Pop: up to 32 nodes from the top of a stack of sibling ranges (first << 3 |
 // count - 1), sp > 0 entries.  Sets v to the lane's node (lanes below the
-// returned count), updates the stack in place.
-__device__ __forceinline__ int bh_pop_nodes(uint32_t* stack, int& sp, unsigned int lt, int& v)
+// returned count) and row to its range's place below the top, updates the
+// stack in place.
+__device__ __forceinline__ int bh_pop_nodes(uint32_t* stack, int& sp, unsigned int lt, int& v, int& row)
 {
     const int lane = threadIdx.x & 31;
     const bool in = lane < sp;
@@ -517,8 +518,8 @@ __device__ __forceinline__ int bh_pop_nodes(uint32_t* stack, int& sp, unsigned i
     const bool begins = in && excl < 32;
     const unsigned int marks = __reduce_or_sync(BH_FULL_MASK, begins ? 1u << (excl & 31) : 0u);
     const int nfull = __popc(__ballot_sync(BH_FULL_MASK, in && excl + c <= 32));
-    const int j = __popc(marks & (lt | (1u << lane))) - 1;
-    v = __shfl_sync(BH_FULL_MASK, st - excl, j) + lane;
+    row = __popc(marks & (lt | (1u << lane))) - 1;
+    v = __shfl_sync(BH_FULL_MASK, st - excl, row) + lane;
     if (begins && lane == nfull) {  // taken in part: the rest stays
         const int take = 32 - excl;
         stack[sp - 1 - lane] = ((uint32_t)(st + take) << 3) | (uint32_t)(c - take - 1);
@@ -528,9 +529,9 @@ __device__ __forceinline__ int bh_pop_nodes(uint32_t* stack, int& sp, unsigned i
 }
 
 // Up to 32 particles from the pending ranges q[pos ..] (n in all).  Returns
-// how many, and the lane's particle in k; advances pos, shortens the range
-// that was taken in part.
-__device__ __forceinline__ int bh_take_particles(int2* q, int& pos, int n, unsigned int lt, int& k)
+// how many, the lane's particle in k and its range's place after pos in row;
+// advances pos, shortens the range that was taken in part.
+__device__ __forceinline__ int bh_take_particles(int2* q, int& pos, int n, unsigned int lt, int& k, int& row)
 {
     const int lane = threadIdx.x & 31;
     const bool in = pos + lane < n;
@@ -547,8 +548,8 @@ __device__ __forceinline__ int bh_take_particles(int2* q, int& pos, int n, unsig
     const bool begins = in && excl < 32;
     const unsigned int marks = __reduce_or_sync(BH_FULL_MASK, begins ? 1u << (excl & 31) : 0u);
     const int nfull = __popc(__ballot_sync(BH_FULL_MASK, in && excl + r.y <= 32));
-    const int j = __popc(marks & (lt | (1u << lane))) - 1;
-    k = __shfl_sync(BH_FULL_MASK, r.x - excl, j) + lane;
+    row = __popc(marks & (lt | (1u << lane))) - 1;
+    k = __shfl_sync(BH_FULL_MASK, r.x - excl, row) + lane;
     if (begins && lane == nfull) q[pos + lane] = make_int2(r.x + (32 - excl), r.y - (32 - excl));
     pos += nfull;
     return min(total, 32);

@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(NW * 32, (T <= 3 ? 16 : 8) / NW) bh_walk_team_
             int4 r;
             auto pop = [&]() -> int {
                 if (sp == 0) return 0;
-                const int npop = bh_pop_nodes(S.stack, sp, lt, v);
+                int row;
+                const int npop = bh_pop_nodes(S.stack, sp, lt, v, row);
                 cm = make_float4(0.f, 0.f, 0.f, 0.f);
                 se = 0.f;
                 r = make_int4(0, 0, -1, 0);

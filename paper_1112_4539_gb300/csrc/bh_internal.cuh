@@ -313,6 +313,32 @@ struct bh_nodes {
 // float4s per walk record (with its padding)
 __host__ __device__ constexpr int bh_wrec_f4(int order) { return order >= 2 ? 5 : 3; }
 
+// ------------------------------------------------- programmatic launch order
+// A kernel launched by bh_launch_after starts while its predecessor in the
+// stream still runs: its blocks come up and then wait in bh_after_previous()
+// until the predecessor has finished and its writes are visible.  Every such
+// kernel calls it before it touches memory that the library or the caller
+// writes, so the order of the stream is kept; bh_let_next_start() allows the
+// successor's blocks to come up.
+__device__ __forceinline__ void bh_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void bh_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t bh_launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
 // --------------------------------------------------------------- launches
 // (bodies in the .cu files; all are stream-ordered and take device pointers)
 namespace bh {

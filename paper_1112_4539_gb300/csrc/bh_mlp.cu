@@ -226,121 +226,273 @@ __global__ void __launch_bounds__(kLabelWarps * 32) bh_mac_label_kernel(LabelArg
 }
 
 // ------------------------------------------------------------ training
-// Activation record per sample: x[6], pre1 mask via h1 > 0, h1[32], h2[32],
-// d1[32] (loss gradient at layer-1 pre-activation), d2[32], dy.
-constexpr int kAct = BH_MLP_NF + 4 * BH_MLP_NH + 1;
 constexpr int kOffB1 = BH_MLP_NH * BH_MLP_NF, kOffW2 = kOffB1 + BH_MLP_NH, kOffB2 = kOffW2 + BH_MLP_NH * BH_MLP_NH,
               kOffW3 = kOffB2 + BH_MLP_NH, kOffB3 = kOffW3 + BH_MLP_NH;
+constexpr int kAct = BH_MLP_NF + 4 * BH_MLP_NH + 1;  // floats of training scratch per sample (caller's buffer)
+constexpr int kRow = BH_MLP_NPARAM + 1;              // a block's partial sums: gradient, loss
+constexpr int kTrainSamples = 64;                    // samples per block and round
+constexpr int kTrainBlocks = 304;                    // most blocks (rows of partial sums)
 
-__global__ void __launch_bounds__(256) bh_mlp_fwd_bwd_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                             const float* __restrict__ Y,
-                                                             const int32_t* __restrict__ order, long long i0, int B,
-                                                             long long n, float under_w, float* __restrict__ act,
-                                                             float* __restrict__ loss, float* __restrict__ yhat)
+// FP32 forward of one sample per thread (training path without gradients).
+__global__ void __launch_bounds__(256) bh_mlp_forward_kernel(const float* __restrict__ P, const float* __restrict__ X,
+                                                             long long i0, int B, float* __restrict__ yhat)
 {
     __shared__ float sp[BH_MLP_NPARAM];
     for (int i = threadIdx.x; i < BH_MLP_NPARAM; i += blockDim.x) sp[i] = P[i];
     __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    const long long s = order ? (long long)order[(i0 + b) % n] : (i0 + b) % n;
-    float x[BH_MLP_NF], h1[BH_MLP_NH], h2[BH_MLP_NH];
-    for (int k = 0; k < BH_MLP_NF; k++) x[k] = X[s * BH_MLP_NF + k];
+    float x[BH_MLP_NF], h1[BH_MLP_NH];
+    for (int k = 0; k < BH_MLP_NF; k++) x[k] = X[(i0 + b) * BH_MLP_NF + k];
+#pragma unroll
     for (int j = 0; j < BH_MLP_NH; j++) {
         float a = sp[kOffB1 + j];
         for (int k = 0; k < BH_MLP_NF; k++) a = fmaf(sp[j * BH_MLP_NF + k], x[k], a);
         h1[j] = fmaxf(a, 0.f);
     }
+    float y = sp[kOffB3];
     for (int j = 0; j < BH_MLP_NH; j++) {
         float a = sp[kOffB2 + j];
+#pragma unroll
         for (int k = 0; k < BH_MLP_NH; k++) a = fmaf(sp[kOffW2 + j * BH_MLP_NH + k], h1[k], a);
-        h2[j] = fmaxf(a, 0.f);
+        y = fmaf(sp[kOffW3 + j], fmaxf(a, 0.f), y);
     }
-    float y = sp[kOffB3];
-    for (int k = 0; k < BH_MLP_NH; k++) y = fmaf(sp[kOffW3 + k], h2[k], y);
-    if (yhat) yhat[b] = y;
-    if (!act) return;
-    const float t = Y[s], r = y - t, wgt = (y < t) ? under_w : 1.0f;
-    if (loss) atomicAdd(loss, wgt * r * r / (float)B);
-    const float dy = 2.0f * wgt * r / (float)B;
-    float* a = act + (size_t)b * kAct;
-    for (int k = 0; k < BH_MLP_NF; k++) a[k] = x[k];
-    float d2[BH_MLP_NH];
-    for (int k = 0; k < BH_MLP_NH; k++) {
-        a[BH_MLP_NF + k] = h1[k];
-        a[BH_MLP_NF + BH_MLP_NH + k] = h2[k];
-        d2[k] = h2[k] > 0.f ? dy * sp[kOffW3 + k] : 0.f;
-        a[BH_MLP_NF + 3 * BH_MLP_NH + k] = d2[k];
-    }
-    for (int k = 0; k < BH_MLP_NH; k++) {
-        float d = 0.f;
-        for (int j = 0; j < BH_MLP_NH; j++) d = fmaf(d2[j], sp[kOffW2 + j * BH_MLP_NH + k], d);
-        a[BH_MLP_NF + 2 * BH_MLP_NH + k] = h1[k] > 0.f ? d : 0.f;
-    }
-    a[kAct - 1] = dy;
+    yhat[b] = y;
 }
 
-// Gradient of the mean loss: block j < 32 reduces hidden unit j's rows of
-// W1, b1, W2, b2 over the batch; block 32 reduces W3 and b3.
-__global__ void __launch_bounds__(256) bh_mlp_grad_kernel(const float* __restrict__ act, int B,
-                                                          float* __restrict__ grad)
+// Forward, backward and the weights' gradient of a mini-batch, 64 samples at
+// a time per block with every activation in shared memory.  Rounds of 64 are
+// dealt to the blocks in turn; a block keeps the gradient sums of its rounds
+// in registers and writes one row of kRow partial sums at the end.  rows == 1
+// (one block): the row is the gradient itself.
+//
+// A step is bound by launches and the latency of its few dependent phases, not
+// by its arithmetic (62 MFLOP for 8192 samples): the activations of a sample
+// used to go through global memory (540 bytes) and 33 blocks read all of them
+// again, each for one unit.  A step of 8192 samples on GB300, 16 steps per call:
+// 127 us (forward and backward 40 us, gradient 82 us, update 4 us), then 20.6 us
+// with this kernel and the sum of its rows, and 13.5 us with each of them
+// launched while its predecessor runs (bh_launch_after).
+struct TrainSmem {
+    float p[BH_MLP_NPARAM + 3];                      // the parameters
+    float w2t[BH_MLP_NH][BH_MLP_NH];                 // W2 transposed: [input][unit]
+    float w2[BH_MLP_NH][BH_MLP_NH];                  // W2: [unit][input]
+    float x[kTrainSamples][BH_MLP_NF + 1];
+    float h1[kTrainSamples][BH_MLP_NH + 1], h2[kTrainSamples][BH_MLP_NH + 1];
+    float d1[kTrainSamples][BH_MLP_NH + 1], d2[kTrainSamples][BH_MLP_NH + 1];
+    float dy[kTrainSamples], l[kTrainSamples];
+};
+
+__global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __restrict__ P,
+                                                                const float* __restrict__ X,
+                                                                const float* __restrict__ Y,
+                                                                const int32_t* __restrict__ order, long long i0, int B,
+                                                                long long n, float under_w, float* __restrict__ rows,
+                                                                float* __restrict__ loss)
 {
-    constexpr int kOut = BH_MLP_NF + 1 + BH_MLP_NH + 1;  // 40 accumulators per thread
-    __shared__ float red[kOut][33];
-    const int j = blockIdx.x;
-    float acc[kOut];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    const int tid = threadIdx.x;
+    bh_let_next_start();
+    // the first round's samples, which no kernel of this call writes, are
+    // fetched before the previous step's parameters are waited for
+    float t = 0.f, x0[BH_MLP_NF];
+    auto fetch = [&](int b) {
+        const bool in = b < B;
+        const long long at = in ? (order ? (long long)order[(i0 + b) % n] : (i0 + b) % n) : 0;
+        t = in ? Y[at] : 0.f;
 #pragma unroll
-    for (int k = 0; k < kOut; k++) acc[k] = 0.f;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        const float* a = act + (size_t)b * kAct;
-        if (j < BH_MLP_NH) {
-            const float d1 = a[BH_MLP_NF + 2 * BH_MLP_NH + j], d2 = a[BH_MLP_NF + 3 * BH_MLP_NH + j];
+        for (int k = 0; k < BH_MLP_NF; k++) x0[k] = in ? X[at * BH_MLP_NF + k] : 0.f;
+    };
+    if (tid < kTrainSamples) fetch(blockIdx.x * kTrainSamples + tid);
+    bh_after_previous();
+    for (int i = tid; i < BH_MLP_NPARAM; i += 256) S.p[i] = P[i];
+    for (int i = tid; i < BH_MLP_NH * BH_MLP_NH; i += 256) {
+        const float w = P[kOffW2 + i];
+        S.w2[i / BH_MLP_NH][i % BH_MLP_NH] = w;
+        S.w2t[i % BH_MLP_NH][i / BH_MLP_NH] = w;
+    }
+    const int s = tid & 63, u0 = (tid >> 6) * 8;  // sample, first of 8 units (a warp shares u0)
+    // weight gradient of layer 2: units ja + 8 a, inputs ka + 8 b, samples q, q + 4, ...
+    const int ja = (tid & 63) >> 3, ka = tid & 7, q = tid >> 6;
+    float g2[4][4];
 #pragma unroll
-            for (int k = 0; k < BH_MLP_NF; k++) acc[k] = fmaf(d1, a[k], acc[k]);
-            acc[BH_MLP_NF] += d1;
+    for (int a = 0; a < 4; a++)
 #pragma unroll
-            for (int k = 0; k < BH_MLP_NH; k++) acc[BH_MLP_NF + 1 + k] = fmaf(d2, a[BH_MLP_NF + k], acc[BH_MLP_NF + 1 + k]);
-            acc[kOut - 1] += d2;
-        } else {
-            const float dy = a[kAct - 1];
+        for (int b = 0; b < 4; b++) g2[a][b] = 0.f;
+    float ge[2] = {0.f, 0.f};  // the thread's one or two other outputs
+    const int nround = (B + kTrainSamples - 1) / kTrainSamples;
+    for (int round = blockIdx.x; round < nround; round += gridDim.x) {
+        const int b = round * kTrainSamples + s;
+        const bool in = b < B;
+        __syncthreads();
+        if (tid < kTrainSamples) {
+            if (round != blockIdx.x) fetch(b);
 #pragma unroll
-            for (int k = 0; k < BH_MLP_NH; k++) acc[k] = fmaf(dy, a[BH_MLP_NF + BH_MLP_NH + k], acc[k]);
-            acc[BH_MLP_NH] += dy;
+            for (int k = 0; k < BH_MLP_NF; k++) S.x[s][k] = x0[k];
+        }
+        __syncthreads();
+        // layer 1
+        {
+            float x[BH_MLP_NF];
+#pragma unroll
+            for (int k = 0; k < BH_MLP_NF; k++) x[k] = S.x[s][k];
+#pragma unroll
+            for (int j = u0; j < u0 + 8; j++) {
+                float a = S.p[kOffB1 + j];
+#pragma unroll
+                for (int k = 0; k < BH_MLP_NF; k++) a = fmaf(S.p[j * BH_MLP_NF + k], x[k], a);
+                S.h1[s][j] = fmaxf(a, 0.f);
+            }
+        }
+        __syncthreads();
+        // layer 2
+        {
+            float a[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) a[j] = S.p[kOffB2 + u0 + j];
+#pragma unroll 8
+            for (int k = 0; k < BH_MLP_NH; k++) {
+                const float h = S.h1[s][k];
+                const float4 w0 = *reinterpret_cast<const float4*>(&S.w2t[k][u0]);
+                const float4 w1 = *reinterpret_cast<const float4*>(&S.w2t[k][u0 + 4]);
+                a[0] = fmaf(w0.x, h, a[0]); a[1] = fmaf(w0.y, h, a[1]); a[2] = fmaf(w0.z, h, a[2]); a[3] = fmaf(w0.w, h, a[3]);
+                a[4] = fmaf(w1.x, h, a[4]); a[5] = fmaf(w1.y, h, a[5]); a[6] = fmaf(w1.z, h, a[6]); a[7] = fmaf(w1.w, h, a[7]);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j++) S.h2[s][u0 + j] = fmaxf(a[j], 0.f);
+        }
+        __syncthreads();
+        // output, loss and its derivative
+        if (tid < kTrainSamples) {
+            float y = S.p[kOffB3];
+#pragma unroll 8
+            for (int k = 0; k < BH_MLP_NH; k++) y = fmaf(S.p[kOffW3 + k], S.h2[s][k], y);
+            const float r = y - t, wgt = (y < t) ? under_w : 1.0f;
+            S.l[s] = in ? wgt * r * r / (float)B : 0.f;
+            S.dy[s] = in ? 2.0f * wgt * r / (float)B : 0.f;
+        }
+        __syncthreads();
+        // back through layer 2 (its derivatives in registers for the thread's 8 units, in memory for all)
+        {
+            const float dy = S.dy[s];
+#pragma unroll
+            for (int j = u0; j < u0 + 8; j++) S.d2[s][j] = S.h2[s][j] > 0.f ? dy * S.p[kOffW3 + j] : 0.f;
+        }
+        __syncthreads();
+        {
+            float d[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) d[k] = 0.f;
+#pragma unroll 8
+            for (int j = 0; j < BH_MLP_NH; j++) {
+                const float e = S.d2[s][j];
+                const float4 w0 = *reinterpret_cast<const float4*>(&S.w2[j][u0]);
+                const float4 w1 = *reinterpret_cast<const float4*>(&S.w2[j][u0 + 4]);
+                d[0] = fmaf(e, w0.x, d[0]); d[1] = fmaf(e, w0.y, d[1]); d[2] = fmaf(e, w0.z, d[2]); d[3] = fmaf(e, w0.w, d[3]);
+                d[4] = fmaf(e, w1.x, d[4]); d[5] = fmaf(e, w1.y, d[5]); d[6] = fmaf(e, w1.z, d[6]); d[7] = fmaf(e, w1.w, d[7]);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; k++) S.d1[s][u0 + k] = S.h1[s][u0 + k] > 0.f ? d[k] : 0.f;
+        }
+        // gradient of W2 (d2 and h1 are complete)
+#pragma unroll 4
+        for (int i = q; i < kTrainSamples; i += 4) {
+            float d[4], h[4];
+#pragma unroll
+            for (int a = 0; a < 4; a++) {
+                d[a] = S.d2[i][ja + 8 * a];
+                h[a] = S.h1[i][ka + 8 * a];
+            }
+#pragma unroll
+            for (int a = 0; a < 4; a++)
+#pragma unroll
+                for (int e = 0; e < 4; e++) g2[a][e] = fmaf(d[a], h[e], g2[a][e]);
+        }
+        __syncthreads();
+        // the other sums: W1 (192), b1 (32), b2 (32); the first 34 threads also W3, b3 and the loss
+        {
+            const float *f, *g;  // columns (stride NH + 1 = 33, or 7 for x)
+            int gs = 0;
+            if (tid < 192) { f = &S.d1[0][tid / BH_MLP_NF]; g = &S.x[0][tid % BH_MLP_NF]; gs = BH_MLP_NF + 1; }
+            else if (tid < 224) { f = &S.d1[0][tid - 192]; g = nullptr; }
+            else { f = &S.d2[0][tid - 224]; g = nullptr; }
+            float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll 8
+            for (int i = 0; i < kTrainSamples; i += 2) {
+                acc0 = fmaf(f[i * (BH_MLP_NH + 1)], g ? g[i * gs] : 1.0f, acc0);
+                acc1 = fmaf(f[(i + 1) * (BH_MLP_NH + 1)], g ? g[(i + 1) * gs] : 1.0f, acc1);
+            }
+            ge[0] += acc0 + acc1;
+            if (tid < BH_MLP_NH + 2) {
+                acc0 = acc1 = 0.f;
+                for (int i = 0; i < kTrainSamples; i += 2) {
+                    const float u = tid < BH_MLP_NH ? S.h2[i][tid] : 1.0f, w = tid < BH_MLP_NH ? S.h2[i + 1][tid] : 1.0f;
+                    acc0 = fmaf(tid == BH_MLP_NH + 1 ? S.l[i] : S.dy[i], u, acc0);
+                    acc1 = fmaf(tid == BH_MLP_NH + 1 ? S.l[i + 1] : S.dy[i + 1], w, acc1);
+                }
+                ge[1] += acc0 + acc1;
+            }
         }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kOut; k++) {
-        float v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(BH_FULL_MASK, v, o);
-        if (lane == 0) red[k][wid] = v;
-    }
+    // the four sample slices of W2's gradient, then the row
     __syncthreads();
-    if (threadIdx.x < kOut) {
-        float v = 0.f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) v += red[threadIdx.x][i];
-        const int k = threadIdx.x;
-        if (j < BH_MLP_NH) {
-            if (k < BH_MLP_NF) grad[j * BH_MLP_NF + k] = v;
-            else if (k == BH_MLP_NF) grad[kOffB1 + j] = v;
-            else if (k < kOut - 1) grad[kOffW2 + j * BH_MLP_NH + (k - BH_MLP_NF - 1)] = v;
-            else grad[kOffB2 + j] = v;
-        } else {
-            if (k < BH_MLP_NH) grad[kOffW3 + k] = v;
-            else if (k == BH_MLP_NH) grad[kOffB3] = v;
-        }
+    float* red = &S.h1[0][0];  // [4][1024] over h1, h2 (4224 floats)
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int e = 0; e < 4; e++) red[q * 1024 + (ja + 8 * a) * BH_MLP_NH + ka + 8 * e] = g2[a][e];
+    __syncthreads();
+    float* row = rows + (size_t)blockIdx.x * (gridDim.x > 1 ? kRow : 0);
+    for (int i = tid; i < 1024; i += 256) row[kOffW2 + i] = (red[i] + red[1024 + i]) + (red[2048 + i] + red[3072 + i]);
+    if (tid < 224) row[tid] = ge[0];              // W1, b1 lie in this order
+    else row[kOffB2 + tid - 224] = ge[0];
+    if (tid < BH_MLP_NH) row[kOffW3 + tid] = ge[1];
+    else if (tid == BH_MLP_NH) row[kOffB3] = ge[1];
+    else if (tid == BH_MLP_NH + 1) {
+        if (gridDim.x > 1) row[BH_MLP_NPARAM] = ge[1];
+        else if (loss) *loss += ge[1];
     }
 }
 
-__global__ void bh_adam_kernel(float* __restrict__ P, const float* __restrict__ g, float* __restrict__ m,
-                               float* __restrict__ v, long long t, float lr, float b1, float b2, float eps)
+// Sum of the rows of partial sums (nrow >= 1), 32 columns per block; then the
+// gradient (grad) or one Adam step (m, v, P).  loss += the rows' losses.
+__global__ void __launch_bounds__(256) bh_mlp_update_kernel(const float* __restrict__ rows, int nrow,
+                                                            float* __restrict__ grad, float* __restrict__ loss,
+                                                            float* __restrict__ P, float* __restrict__ m,
+                                                            float* __restrict__ v, long long t, float lr, float b1,
+                                                            float b2, float eps)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= BH_MLP_NPARAM) return;
+    __shared__ float red[8][33];
+    const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + c;
+    bh_let_next_start();
+    bh_after_previous();
+    float a0 = 0.f, a1 = 0.f;
+    if (k < (nrow > 1 ? kRow : BH_MLP_NPARAM)) {  // (a single row is a bare gradient)
+        int r = w;
+#pragma unroll 8
+        for (; r + 8 < nrow; r += 16) {
+            a0 += rows[(size_t)r * kRow + k];
+            a1 += rows[(size_t)(r + 8) * kRow + k];
+        }
+        if (r < nrow) a0 += rows[(size_t)r * kRow + k];
+    }
+    red[w][c] = a0 + a1;
+    __syncthreads();
+    if (w != 0 || k >= kRow) return;
+    float g = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; i++) g += red[i][c];
+    if (k == BH_MLP_NPARAM) {
+        if (loss && nrow > 1) *loss += g;
+        return;
+    }
+    if (grad) grad[k] = g;
+    if (!P) return;
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    const float mk = b1 * m[k] + (1.f - b1) * g[k];
-    const float vk = b2 * v[k] + (1.f - b2) * g[k] * g[k];
+    const float mk = b1 * m[k] + (1.f - b1) * g;
+    const float vk = b2 * v[k] + (1.f - b2) * g * g;
     m[k] = mk;
     v[k] = vk;
     P[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
@@ -435,6 +587,12 @@ int mac_label(const float4* pos_s, const uint32_t* perm, const int32_t* g_first,
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
 
+static bool train_smem_ok()
+{
+    return cudaFuncSetAttribute(bh_mlp_batch_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(TrainSmem)) == cudaSuccess;
+}
+
 int mlp_train(const float* X, const float* Y, const int32_t* order, long long n, float* P, float* adam_m,
               float* adam_v, float* work, long long work_floats, long long steps, int batch, float lr,
               float under_w, float* loss, long long t0, cudaStream_t s)
@@ -442,16 +600,19 @@ int mlp_train(const float* X, const float* Y, const int32_t* order, long long n,
     if (batch < 1 || n < 1 || steps < 0) return BH_ERR_INVALID;
     const long long need = (long long)batch * kAct + BH_MLP_NPARAM;
     if (work_floats < need) return BH_ERR_TOO_LARGE;
-    float* act = work;
-    float* grad = work + (size_t)batch * kAct;
-    const int blocks = (batch + 255) / 256;
+    const int blocks = std::min((batch + kTrainSamples - 1) / kTrainSamples, kTrainBlocks);
+    if (!train_smem_ok()) return BH_ERR_CUDA;
     for (long long st = 0; st < steps; st++) {
         const long long i0 = ((t0 + st) * (long long)batch) % n;
-        bh_mlp_fwd_bwd_kernel<<<blocks, 256, 0, s>>>(P, X, Y, order, i0, batch, n, under_w, act,
-                                                     loss ? loss + st : nullptr, nullptr);
-        bh_mlp_grad_kernel<<<BH_MLP_NH + 1, 256, 0, s>>>(act, batch, grad);
-        bh_adam_kernel<<<(BH_MLP_NPARAM + 255) / 256, 256, 0, s>>>(P, grad, adam_m, adam_v, t0 + st + 1, lr, 0.9f,
-                                                                   0.999f, 1e-8f);
+        float* l = loss ? loss + st : nullptr;
+        if (st == 0)  // its samples may still be in the making
+            bh_mlp_batch_grad_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, X, Y, order, i0, batch, n, under_w, work,
+                                                                            l);
+        else
+            bh_launch_after(bh_mlp_batch_grad_kernel, blocks, 256, sizeof(TrainSmem), s, P, X, Y, order, i0, batch, n,
+                            under_w, work, l);
+        bh_launch_after(bh_mlp_update_kernel, (kRow + 31) / 32, 256, 0, s, work, blocks, nullptr, l, P, adam_m, adam_v,
+                        t0 + st + 1, lr, 0.9f, 0.999f, 1e-8f);
     }
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
@@ -462,9 +623,14 @@ int mlp_grad(const float* P, const float* X, const float* Y, long long n, float 
     const long long need = n * kAct;
     if (work_floats < need) return BH_ERR_TOO_LARGE;
     if (n > (1ll << 30)) return BH_ERR_TOO_LARGE;
-    bh_mlp_fwd_bwd_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(P, X, Y, nullptr, 0, (int)n, n, under_w, work, loss,
-                                                                 nullptr);
-    bh_mlp_grad_kernel<<<BH_MLP_NH + 1, 256, 0, s>>>(work, (int)n, grad);
+    // rows of partial sums fit in n * kAct floats whenever there are two or more (n > 64)
+    const int blocks = (int)std::min<long long>((n + kTrainSamples - 1) / kTrainSamples, kTrainBlocks);
+    if (!train_smem_ok()) return BH_ERR_CUDA;
+    bh_mlp_batch_grad_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, X, Y, nullptr, 0, (int)n, n, under_w,
+                                                                    blocks > 1 ? work : grad, loss);
+    if (blocks > 1)
+        bh_mlp_update_kernel<<<(kRow + 31) / 32, 256, 0, s>>>(work, blocks, grad, loss, nullptr, nullptr, nullptr, 1,
+                                                              0.f, 0.9f, 0.999f, 1e-8f);
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
 
@@ -478,8 +644,7 @@ int mlp_forward(const float* P, const bh_mlp_dev* Wdev, const float* X, long lon
         // FP32 training forward, in chunks the kernel's int batch can index
         for (long long i0 = 0; i0 < n; i0 += (1ll << 30)) {
             const int B = (int)std::min<long long>(n - i0, 1ll << 30);
-            bh_mlp_fwd_bwd_kernel<<<(B + 255) / 256, 256, 0, s>>>(P, X, nullptr, nullptr, i0, B, n, 1.f, nullptr,
-                                                                  nullptr, y + i0);
+            bh_mlp_forward_kernel<<<(B + 255) / 256, 256, 0, s>>>(P, X, i0, B, y + i0);
         }
     }
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;

@@ -301,8 +301,8 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
         bh::launch_keys(pos, N, x->ctrl, x->keys, x->cfg.curve, x->deep, grid_for(x), s);
         bh::launch_sort(x->keys, x->keys_alt, x->vals, x->vals_alt, pos, x->pos_s, N, x->lookback, x->ctrl,
                         x->deep, s);
-        bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->nd, x->node_cap, x->ctrl,
-                        grid_for(x), s);
+        bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap,
+                        x->ctrl, grid_for(x), s);
         bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, x->ctrl,
                           grid_for(x), s);
         x->launches += bh::launches_build(x->deep) - 1;
@@ -743,8 +743,8 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     bh::launch_init(x->ctrl, s);
     bh::launch_batch_sort((const float4*)d_pos_mass, x->sys_off, x->nsys, x->keys, x->keys_alt, x->vals, x->vals_alt,
                           x->pos_s, x->sys_of, x->sys_box, x->cfg.curve, x->deep, x->ctrl, s);
-    bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->nd, x->node_cap, x->ctrl, grid_for(x),
-                    s, x->sys_of, x->sys_off);
+    bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap, x->ctrl,
+                    grid_for(x), s, x->sys_of, x->sys_off);
     bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, x->ctrl, grid_for(x), s);
     bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
                        x->cfg.curve, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
@@ -752,8 +752,8 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
                              (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
-    // init, batch sort, 4 tree, 5 groups, moments per level, 2 walk
-    x->launches += 2 + 4 + 5 + bh::launches_moments(x->deep) + bh::kLaunchesForce;
+    // init, batch sort, 4 tree, 3 groups, moments per level, 2 walk
+    x->launches += 2 + 4 + 3 + bh::launches_moments(x->deep) + bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
     x->theta = theta;

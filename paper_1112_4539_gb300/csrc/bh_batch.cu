@@ -24,6 +24,8 @@ bh_batch_sort_kernel(const float4* __restrict__ pos, const int32_t* __restrict__
                      K* keys_alt, uint32_t* vals, uint32_t* vals_alt, float4* __restrict__ pos_s,
                      uint32_t* __restrict__ sys, float4* __restrict__ sys_box, bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous(pos, off, pos_s, sys, sys_box);
     constexpr int B = bh_key_traits<K>::kMaxLevel, NP = bh_key_traits<K>::kPasses;
     constexpr unsigned int CMAX = (1u << B) - 1u;
     __shared__ unsigned int whist[kBWarps][256];
@@ -183,10 +185,10 @@ void launch_batch_sort(const float4* pos, const int32_t* sys_off, int nsys, void
 {
     if (nsys <= 0) return;
     if (deep)
-        bh_batch_sort_kernel<bh_key64><<<nsys, kBT, 0, s>>>(pos, sys_off, curve, (bh_key64*)keys, (bh_key64*)keys_alt,
+        bh_launch_after(bh_batch_sort_kernel<bh_key64>, nsys, kBT, 0, s, pos, sys_off, curve, (bh_key64*)keys, (bh_key64*)keys_alt,
                                                             vals, vals_alt, pos_s, sys, sys_box, ctrl);
     else
-        bh_batch_sort_kernel<uint32_t><<<nsys, kBT, 0, s>>>(pos, sys_off, curve, (uint32_t*)keys, (uint32_t*)keys_alt,
+        bh_launch_after(bh_batch_sort_kernel<uint32_t>, nsys, kBT, 0, s, pos, sys_off, curve, (uint32_t*)keys, (uint32_t*)keys_alt,
                                                             vals, vals_alt, pos_s, sys, sys_box, ctrl);
 }
 

@@ -320,7 +320,20 @@ __host__ __device__ constexpr int bh_wrec_f4(int order) { return order >= 2 ? 5 
 // kernel calls it before it touches memory that the library or the caller
 // writes, so the order of the stream is kept; bh_let_next_start() allows the
 // successor's blocks to come up.
-__device__ __forceinline__ void bh_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class T>
+__device__ __forceinline__ void bh_reload(T& p)
+{
+    asm volatile("" : "+l"(p));
+}
+// p: the kernel's __restrict__ pointers.  Loads through such a pointer may be
+// taken for loads of constant memory and moved over the wait; the pointers
+// are made unknown after it, which ties every load to its place.
+template <class... T>
+__device__ __forceinline__ void bh_after_previous(T&... p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (bh_reload(p), ...);
+}
 __device__ __forceinline__ void bh_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
@@ -364,7 +377,8 @@ void launch_sort(void* keys, void* keys_alt, uint32_t* vals, uint32_t* vals_alt,
 // Morton position, first particle of each system + total, root cube of each);
 // null for a single system.
 // dl: uint16_t[n] scratch; blk_lvl: (deepest level + 1) * ceil(n / kLevelTile) words
-void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl,
+// flags: cleared for launch_groups (padded to whole kFlagTile blocks)
+void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, uint8_t* flags,
                  const bh_nodes& nd, int64_t node_cap, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                  const uint32_t* sys = nullptr, const int32_t* sys_off = nullptr);
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
@@ -419,7 +433,7 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
                float* rho, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
 
 // launches per call (deep = 63-bit keys: 8 sort passes, 22 levels)
-inline int launches_build(bool deep) { return deep ? 20 : 16; }  // init, bbox, keys, sort passes, 4 tree, 5 groups
+inline int launches_build(bool deep) { return deep ? 18 : 14; }  // init, bbox, keys, sort passes, 4 tree, 3 groups
 inline int launches_moments(bool deep) { return (deep ? 22 : 11) + 1; }  // large leaves, one per level
 constexpr int kLaunchesForce = 2;    // counter reset, walk
 constexpr int kLaunchesPWalk = 4;    // parent links, next links, counter reset, walk

@@ -8,6 +8,8 @@ __global__ void __launch_bounds__(256) bh_kick_drift_kernel(float4* __restrict__
                                                             const float4* __restrict__ acc, int n, float dt_kick,
                                                             float dt_drift)
 {
+    bh_let_next_start();
+    bh_after_previous(pos, vel, acc);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float4 a = acc[i];
         float4 v = vel[i];
@@ -27,7 +29,7 @@ void launch_kick_drift(float4* pos, float4* vel, const float4* acc, int n, float
                        cudaStream_t s)
 {
     if (n <= 0) return;
-    bh_kick_drift_kernel<<<grid, 256, 0, s>>>(pos, vel, acc, n, dt_kick, dt_drift);
+    bh_launch_after(bh_kick_drift_kernel, grid, 256, 0, s, pos, vel, acc, n, dt_kick, dt_drift);
 }
 
 }  // namespace bh

@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
         for (int k = 0; k < BH_MLP_NF; k++) x0[k] = in ? X[at * BH_MLP_NF + k] : 0.f;
     };
     if (tid < kTrainSamples) fetch(blockIdx.x * kTrainSamples + tid);
-    bh_after_previous();
+    bh_after_previous(P, rows, loss);
     for (int i = tid; i < BH_MLP_NPARAM; i += 256) S.p[i] = P[i];
     for (int i = tid; i < BH_MLP_NH * BH_MLP_NH; i += 256) {
         const float w = P[kOffW2 + i];
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(256) bh_mlp_update_kernel(const float* __restr
     const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + c;
     bh_let_next_start();
-    bh_after_previous();
+    bh_after_previous(rows, grad, loss, P, m, v);
     float a0 = 0.f, a1 = 0.f;
     if (k < (nrow > 1 ? kRow : BH_MLP_NPARAM)) {  // (a single row is a bare gradient)
         int r = w;

@@ -28,6 +28,8 @@ constexpr int kLinkDepthCap = 32;  // > the 22 levels of a 63-bit key tree
 __global__ void bh_parent_kernel(const int4* __restrict__ rec, int32_t* __restrict__ parent,
                                  const bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(rec, parent, c);
     const int nn = (int)c->n_nodes, n_roots = (int)c->level_offset[1];
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nn; v += gridDim.x * blockDim.x) {
         const int4 r = rec[v];
@@ -40,6 +42,8 @@ __global__ void bh_parent_kernel(const int4* __restrict__ rec, int32_t* __restri
 __global__ void bh_next_kernel(const int4* __restrict__ rec, const int32_t* __restrict__ parent,
                                int32_t* __restrict__ next, bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(rec, parent, next, c);
     const int nn = (int)c->n_nodes;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nn; v += gridDim.x * blockDim.x) {
         int u = v, nx = -1, d = 0;
@@ -215,6 +219,8 @@ __device__ __forceinline__ void bh_p_put(float4* a, float4* b, float4* c, int r,
 template <int ORDER, bool IND, bool NORMAL>
 __global__ void __launch_bounds__(kPThreads, 5) bh_pwalk_kernel(PWalkParams P, int stack_cap)
 {
+    bh_let_next_start();
+    bh_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef PSmem<ORDER, IND> Smem;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -423,6 +429,8 @@ __global__ void __launch_bounds__(kPThreads, 5) bh_pwalk_kernel(PWalkParams P, i
 
 __global__ void bh_pwalk_reset_kernel(bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous();
     c->group_ctr = 0u;
     c->n_pp = 0ull;
     c->n_pc = 0ull;
@@ -434,6 +442,8 @@ __global__ void __launch_bounds__(256) bh_soft_gather_kernel(const float* __rest
                                                              const uint32_t* __restrict__ perm, int n,
                                                              float* __restrict__ h, bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous(eps, perm, h);
     bool bad = false;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const float e = eps[perm[k]];
@@ -450,6 +460,8 @@ __global__ void __launch_bounds__(256) bh_soft_level_kernel(const float4* __rest
                                                             double2* __restrict__ sums, float* __restrict__ hbar,
                                                             const bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(pos_s, h, sums, hbar, c);
     if (c->n_nodes == 0u) return;
     const int v0 = (int)c->level_offset[lev], v1 = (int)c->level_offset[lev + 1];
     for (int v = v0 + blockIdx.x * blockDim.x + threadIdx.x; v < v1; v += gridDim.x * blockDim.x) {
@@ -476,9 +488,9 @@ __global__ void __launch_bounds__(256) bh_soft_level_kernel(const float4* __rest
 void launch_softening(const float* eps, const uint32_t* perm, const float4* pos_s, const bh_nodes& nd, int n,
                       bool deep, const bh_soft& soft, bh_dev_ctrl* ctrl, int grid, cudaStream_t s)
 {
-    bh_soft_gather_kernel<<<grid, 256, 0, s>>>(eps, perm, n, soft.h, ctrl);
+    bh_launch_after(bh_soft_gather_kernel, grid, 256, 0, s, eps, perm, n, soft.h, ctrl);
     for (int lev = deep ? BH_MAX_LEVEL_DEEP : BH_MAX_LEVEL; lev >= 0; lev--)
-        bh_soft_level_kernel<<<grid, 256, 0, s>>>(pos_s, soft.h, nd, lev, soft.sums, soft.hbar, ctrl);
+        bh_launch_after(bh_soft_level_kernel, grid, 256, 0, s, pos_s, soft.h, nd, lev, soft.sums, soft.hbar, ctrl);
 }
 
 // persistent warps, as many blocks per SM as registers and shared memory allow;
@@ -494,7 +506,7 @@ static int bh_pwalk_launch(const PWalkParams& P, bool deep, int sm_count, cudaSt
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPThreads, smem) != cudaSuccess || bps < 1)
         return BH_ERR_CUDA;
     const int warps = (P.n + 31) / 32, blocks = (warps + kPThreads / 32 - 1) / (kPThreads / 32);
-    kern<<<std::min(blocks, sm_count * bps), kPThreads, smem, s>>>(P, cap);
+    bh_launch_after(kern, std::min(blocks, sm_count * bps), kPThreads, smem, s, P, cap);
     return BH_OK;
 }
 
@@ -503,9 +515,9 @@ int launch_pwalk(const float4* pos_s, const uint32_t* perm, const bh_nodes& nd, 
                  int sm_count, cudaStream_t s, const bh_soft* soft)
 {
     const int link_grid = std::max(1, std::min((node_cap + 255) / 256, sm_count * 16));
-    bh_parent_kernel<<<link_grid, 256, 0, s>>>(nd.rec, parent, ctrl);
-    bh_next_kernel<<<link_grid, 256, 0, s>>>(nd.rec, parent, next, ctrl);
-    bh_pwalk_reset_kernel<<<1, 1, 0, s>>>(ctrl);
+    bh_launch_after(bh_parent_kernel, link_grid, 256, 0, s, nd.rec, parent, ctrl);
+    bh_launch_after(bh_next_kernel, link_grid, 256, 0, s, nd.rec, parent, next, ctrl);
+    bh_launch_after(bh_pwalk_reset_kernel, 1, 1, 0, s, ctrl);
     PWalkParams P;
     P.pos_s = pos_s;
     P.perm = perm;

@@ -16,6 +16,8 @@ namespace bh {
 
 __global__ void bh_init_kernel(bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous();
     const int t = threadIdx.x;
     if (t < 3) {
         c->minmax[t] = 0xffffffffu;
@@ -42,11 +44,13 @@ __global__ void bh_init_kernel(bh_dev_ctrl* c)
     }
 }
 
-void launch_init(bh_dev_ctrl* ctrl, cudaStream_t s) { bh_init_kernel<<<1, 256, 0, s>>>(ctrl); }
+void launch_init(bh_dev_ctrl* ctrl, cudaStream_t s) { bh_launch_after(bh_init_kernel, 1, 256, 0, s, ctrl); }
 
 // Per-axis min/max over all particles; flags NaN/Inf coordinates or masses.
 __global__ void __launch_bounds__(256) bh_bbox_kernel(const float4* __restrict__ pos, int n, bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous(pos);
     unsigned int lo0 = 0xffffffffu, lo1 = 0xffffffffu, lo2 = 0xffffffffu, hi0 = 0u, hi1 = 0u, hi2 = 0u;
     bool bad = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -97,7 +101,7 @@ __global__ void __launch_bounds__(256) bh_bbox_kernel(const float4* __restrict__
 
 void launch_bbox(const float4* pos, int n, bh_dev_ctrl* ctrl, int grid, cudaStream_t s)
 {
-    bh_bbox_kernel<<<grid, 256, 0, s>>>(pos, n, ctrl);
+    bh_launch_after(bh_bbox_kernel, grid, 256, 0, s, pos, n, ctrl);
 }
 
 // ------------------------------------------------------------------ keys
@@ -109,6 +113,8 @@ template <int CURVE, typename K>
 __global__ void __launch_bounds__(256) bh_keys_kernel(const float4* __restrict__ pos, int n, bh_dev_ctrl* c,
                                                       K* __restrict__ keys)
 {
+    bh_let_next_start();
+    bh_after_previous(pos, keys);
     constexpr int B = bh_key_traits<K>::kMaxLevel, NP = bh_key_traits<K>::kPasses;
     constexpr unsigned int CMAX = (1u << B) - 1u;
     __shared__ unsigned int sh[NP][256];
@@ -150,12 +156,12 @@ void launch_keys(const float4* pos, int n, bh_dev_ctrl* ctrl, void* keys, int cu
 {
     if (deep) {
         bh_key64* k = (bh_key64*)keys;
-        if (curve == BH_CURVE_HILBERT) bh_keys_kernel<BH_CURVE_HILBERT, bh_key64><<<grid, 256, 0, s>>>(pos, n, ctrl, k);
-        else bh_keys_kernel<BH_CURVE_MORTON, bh_key64><<<grid, 256, 0, s>>>(pos, n, ctrl, k);
+        if (curve == BH_CURVE_HILBERT) bh_launch_after(bh_keys_kernel<BH_CURVE_HILBERT, bh_key64>, grid, 256, 0, s, pos, n, ctrl, k);
+        else bh_launch_after(bh_keys_kernel<BH_CURVE_MORTON, bh_key64>, grid, 256, 0, s, pos, n, ctrl, k);
     } else {
         uint32_t* k = (uint32_t*)keys;
-        if (curve == BH_CURVE_HILBERT) bh_keys_kernel<BH_CURVE_HILBERT, uint32_t><<<grid, 256, 0, s>>>(pos, n, ctrl, k);
-        else bh_keys_kernel<BH_CURVE_MORTON, uint32_t><<<grid, 256, 0, s>>>(pos, n, ctrl, k);
+        if (curve == BH_CURVE_HILBERT) bh_launch_after(bh_keys_kernel<BH_CURVE_HILBERT, uint32_t>, grid, 256, 0, s, pos, n, ctrl, k);
+        else bh_launch_after(bh_keys_kernel<BH_CURVE_MORTON, uint32_t>, grid, 256, 0, s, pos, n, ctrl, k);
     }
 }
 
@@ -263,6 +269,8 @@ bh_onesweep_kernel(const K* __restrict__ kin, const uint32_t* __restrict__ vin, 
                    uint32_t* __restrict__ vout, const float4* __restrict__ pos, float4* __restrict__ pos_s, int n,
                    int shift, int pass, unsigned long long* lookback, bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous(kin, vin, kout, vout, pos, pos_s);
     const unsigned int epoch = c->build_seq * 8u + (unsigned int)pass + 1u;
     constexpr int W = THREADS / 32;
     constexpr int ITEMS = TILE / THREADS;
@@ -404,14 +412,11 @@ static void bh_sort_passes(K* keys, K* keys_alt, uint32_t* vals, uint32_t* vals_
     uint32_t *va = vals, *vb = vals_alt;
     for (int p = 0; p < NP; p++) {
         if (p == 0)
-            bh_onesweep_kernel<K, TILE, THREADS0, true, false>
-                <<<tiles, THREADS0, 0, s>>>(ka, nullptr, kb, vb, pos, pos_s, n, 0, 0, lookback, ctrl);
+            bh_launch_after(bh_onesweep_kernel<K, TILE, THREADS0, true, false>, tiles, THREADS0, 0, s, ka, nullptr, kb, vb, pos, pos_s, n, 0, 0, lookback, ctrl);
         else if (p == NP - 1)
-            bh_onesweep_kernel<K, TILE, THREADS, false, true>
-                <<<tiles, THREADS, 0, s>>>(ka, va, kb, vb, pos, pos_s, n, 8 * p, p, lookback, ctrl);
+            bh_launch_after(bh_onesweep_kernel<K, TILE, THREADS, false, true>, tiles, THREADS, 0, s, ka, va, kb, vb, pos, pos_s, n, 8 * p, p, lookback, ctrl);
         else
-            bh_onesweep_kernel<K, TILE, THREADS, false, false>
-                <<<tiles, THREADS, 0, s>>>(ka, va, kb, vb, pos, pos_s, n, 8 * p, p, lookback, ctrl);
+            bh_launch_after(bh_onesweep_kernel<K, TILE, THREADS, false, false>, tiles, THREADS, 0, s, ka, va, kb, vb, pos, pos_s, n, 8 * p, p, lookback, ctrl);
         K* tk = ka; ka = kb; kb = tk;
         uint32_t* tv = va; va = vb; vb = tv;
     }

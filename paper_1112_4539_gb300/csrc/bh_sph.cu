@@ -39,6 +39,8 @@ __global__ void bh_node_box_kernel(const float4* __restrict__ pos_s, const int4*
                                    float4* __restrict__ lo, float4* __restrict__ hi, int lev,
                                    const bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(pos_s, rec, lo, hi, c);
     const int v0 = (int)c->level_offset[lev], v1 = (int)c->level_offset[lev + 1];
     for (int v = v0 + blockIdx.x * blockDim.x + threadIdx.x; v < v1; v += gridDim.x * blockDim.x) {
         const int4 r = rec[v];
@@ -122,6 +124,8 @@ __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ src, cons
 template <int T>
 __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
 {
+    bh_let_next_start();
+    bh_after_previous();
     __shared__ SphSmem smem[4];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     SphSmem& S = smem[wib];
@@ -348,6 +352,8 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
 
 __global__ void bh_sph_reset_kernel(bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous();
     c->group_ctr = 0u;
     c->n_pp = 0ull;
     c->n_pc = 0ull;
@@ -362,7 +368,7 @@ static int bh_sph_launch(const SphParams& P, int sm_count, cudaStream_t s)
         cudaGetLastError();
         bps = 4;
     }
-    bh_sph_kernel<T><<<sm_count * bps, 128, 0, s>>>(P);
+    bh_launch_after(bh_sph_kernel<T>, sm_count * bps, 128, 0, s, P);
     return BH_OK;
 }
 
@@ -371,8 +377,8 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
                float* rho, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s)
 {
     for (int lev = max_level; lev >= 0; lev--)
-        bh_node_box_kernel<<<grid, 256, 0, s>>>(pos_s, nd.rec, blo, bhi, lev, ctrl);
-    bh_sph_reset_kernel<<<1, 1, 0, s>>>(ctrl);
+        bh_launch_after(bh_node_box_kernel, grid, 256, 0, s, pos_s, nd.rec, blo, bhi, lev, ctrl);
+    bh_launch_after(bh_sph_reset_kernel, 1, 1, 0, s, ctrl);
     SphParams P;
     P.pos_s = pos_s;
     P.perm = perm;

@@ -171,8 +171,8 @@ extern "C" int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh
     bh::launch_keys(pos, N32, ctrl, keys, c.curve, false, grid, s);
     bh::launch_sort(keys, keys_alt, vals, vals_alt, pos, pos_s, N32, (unsigned long long*)(b + o_look), ctrl,
                     false, s);
-    bh::launch_tree(keys, false, N32, c.leaf_size, (uint16_t*)(b + o_dl), (uint32_t*)(b + o_blk), nd, (int64_t)NN,
-                    ctrl, grid, s);
+    bh::launch_tree(keys, false, N32, c.leaf_size, (uint16_t*)(b + o_dl), (uint32_t*)(b + o_blk),
+                    (uint8_t*)(b + o_flags), nd, (int64_t)NN, ctrl, grid, s);
     bh::launch_groups(nd, N32, c.group_size, (uint8_t*)(b + o_flags), (uint32_t*)(b + o_blk), g_first, g_count,
                       ctrl, grid, s);
     bh::launch_moments(pos_s, keys, false, nd, c.order, theta, c.fp64_node_threshold, c.curve, ctrl, grid, s);

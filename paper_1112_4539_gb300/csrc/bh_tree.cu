@@ -39,8 +39,10 @@ constexpr int kWarpMomentLevels = BH_WARP_MOMENT_LEVELS;  // levels 0..this: a w
 template <typename K>
 __global__ void __launch_bounds__(kLvlThreads)
 bh_levels_kernel(const K* __restrict__ keys, const uint32_t* __restrict__ sys, int n, int n_leaf,
-                 uint16_t* __restrict__ dl, uint32_t* __restrict__ blk_lvl, int nblk)
+                 uint16_t* __restrict__ dl, uint32_t* __restrict__ blk_lvl, int nblk, uint8_t* __restrict__ flags)
 {
+    bh_let_next_start();
+    bh_after_previous(keys, sys, dl, blk_lvl, flags);
     constexpr int L = bh_key_traits<K>::kMaxLevel;
     __shared__ K sk[kLevelTile + 2 * kMaxLeaf + 2];
     __shared__ uint32_t ss[kLevelTile + 2 * kMaxLeaf + 2];
@@ -49,6 +51,9 @@ bh_levels_kernel(const K* __restrict__ keys, const uint32_t* __restrict__ sys, i
     const int tid = threadIdx.x;
     const int base = blockIdx.x * kLevelTile;
     if (tid <= L) sblk[tid] = 0u;
+    // clear the group flags of the block's positions (8 per thread; the array is padded to whole blocks)
+    static_assert(kLvlPer == 8 && kFlagTile % kLevelTile == 0, "8 flags per thread, whole blocks of flags");
+    *reinterpret_cast<uint2*>(flags + base + 8 * tid) = make_uint2(0u, 0u);
     const int lo = base - n_leaf - 1;
     const int span = kLevelTile + 2 * n_leaf + 1;
     for (int i = tid; i < span; i += kLvlThreads) {
@@ -168,6 +173,8 @@ __device__ unsigned int bh_scan_segment(uint32_t* a, int len, unsigned int* wtot
 __global__ void __launch_bounds__(1024) bh_level_scan_kernel(uint32_t* blk_lvl, int nblk, int nlev, bh_dev_ctrl* c,
                                                              long long node_cap)
 {
+    bh_let_next_start();
+    bh_after_previous();
     __shared__ unsigned int wtot[33];
     __shared__ bool last;
     const int l = blockIdx.x;
@@ -206,6 +213,8 @@ bh_node_write_kernel(const uint16_t* __restrict__ dl, int n, const uint32_t* __r
                      const bh_dev_ctrl* __restrict__ c, int32_t* __restrict__ nfirst, uint8_t* __restrict__ nlevel,
                      int32_t* __restrict__ nchildidx)
 {
+    bh_let_next_start();
+    bh_after_previous(dl, blk_lvl, c, nfirst, nlevel, nchildidx);
     __shared__ unsigned int swt[kLvlThreads / 32][L + 1];
     __shared__ unsigned int sx[L + 1][kLvlThreads];  // per level and thread: count, then next node index
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -264,6 +273,8 @@ __global__ void __launch_bounds__(256)
 bh_node_finalize_kernel(const K* __restrict__ keys, const uint32_t* __restrict__ sys,
                         const int32_t* __restrict__ sys_off, int n, bh_nodes nd, bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous(keys, sys, sys_off);
     constexpr int L = bh_key_traits<K>::kMaxLevel;
     const int nn = (int)c->n_nodes;
     unsigned int leaves = 0u, maxleaf = 0u;
@@ -314,27 +325,30 @@ bh_node_finalize_kernel(const K* __restrict__ keys, const uint32_t* __restrict__
 }
 
 template <typename K>
-static void bh_tree_t(const K* keys, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, const bh_nodes& nd,
+static void bh_tree_t(const K* keys, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, uint8_t* flags, const bh_nodes& nd,
                       int64_t node_cap, bh_dev_ctrl* ctrl, int grid, cudaStream_t s, const uint32_t* sys,
                       const int32_t* sys_off)
 {
     constexpr int L = bh_key_traits<K>::kMaxLevel;
     const int nblk = (n + kLevelTile - 1) / kLevelTile;
-    bh_levels_kernel<K><<<nblk, kLvlThreads, 0, s>>>(keys, sys, n, n_leaf, dl, blk_lvl, nblk);
-    bh_level_scan_kernel<<<L + 1, 1024, 0, s>>>(blk_lvl, nblk, L + 1, ctrl, (long long)node_cap);
-    bh_node_write_kernel<L><<<nblk, kLvlThreads, 0, s>>>(dl, n, blk_lvl, nblk, ctrl, nd.first, nd.level, nd.child);
-    bh_node_finalize_kernel<K><<<grid, 256, 0, s>>>(keys, sys, sys_off, n, nd, ctrl);
+    bh_launch_after(bh_levels_kernel<K>, nblk, kLvlThreads, 0, s, keys, sys, n, n_leaf, dl, blk_lvl, nblk, flags);
+    bh_launch_after(bh_level_scan_kernel, L + 1, 1024, 0, s, blk_lvl, nblk, L + 1, ctrl, (long long)node_cap);
+    bh_launch_after(bh_node_write_kernel<L>, nblk, kLvlThreads, 0, s, dl, n, blk_lvl, nblk, ctrl, nd.first, nd.level, nd.child);
+    bh_launch_after(bh_node_finalize_kernel<K>, grid, 256, 0, s, keys, sys, sys_off, n, nd, ctrl);
 }
 
-void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, const bh_nodes& nd,
+void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, uint8_t* flags,
+                 const bh_nodes& nd,
                  int64_t node_cap, bh_dev_ctrl* ctrl, int grid, cudaStream_t s, const uint32_t* sys,
                  const int32_t* sys_off)
 {
     if (n <= 0) return;
     if (deep)
-        bh_tree_t<bh_key64>((const bh_key64*)keys, n, n_leaf, dl, blk_lvl, nd, node_cap, ctrl, grid, s, sys, sys_off);
+        bh_tree_t<bh_key64>((const bh_key64*)keys, n, n_leaf, dl, blk_lvl, flags, nd, node_cap, ctrl, grid, s, sys,
+                            sys_off);
     else
-        bh_tree_t<uint32_t>((const uint32_t*)keys, n, n_leaf, dl, blk_lvl, nd, node_cap, ctrl, grid, s, sys, sys_off);
+        bh_tree_t<uint32_t>((const uint32_t*)keys, n, n_leaf, dl, blk_lvl, flags, nd, node_cap, ctrl, grid, s, sys,
+                            sys_off);
 }
 
 // ------------------------------------------------------------ groups
@@ -345,6 +359,8 @@ void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, u
 __global__ void __launch_bounds__(256) bh_group_mark_kernel(bh_nodes nd, int G, uint8_t* __restrict__ flags,
                                                             const bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(flags, c);
     const int nn = (int)c->n_nodes;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nn; v += gridDim.x * blockDim.x) {
         const int4 r = nd.rec[v];
@@ -383,6 +399,8 @@ constexpr int kFlagPer = kFlagTile / kFlagThreads;  // 16 bytes per thread
 __global__ void __launch_bounds__(kFlagThreads) bh_flag_count_kernel(const uint8_t* __restrict__ flags, int n,
                                                                      uint32_t* __restrict__ blk)
 {
+    bh_let_next_start();
+    bh_after_previous(flags, blk);
     __shared__ unsigned int ws[kFlagThreads / 32];
     const int base = blockIdx.x * kFlagTile + threadIdx.x * kFlagPer;
     unsigned int s = 0u;
@@ -402,49 +420,77 @@ __global__ void __launch_bounds__(kFlagThreads) bh_flag_count_kernel(const uint8
     }
 }
 
-__global__ void __launch_bounds__(1024) bh_flag_scan_kernel(uint32_t* blk, int nblk, bh_dev_ctrl* c)
-{
-    __shared__ unsigned int wtot[33];
-    const unsigned int t = bh_scan_segment(blk, nblk, wtot);
-    if (threadIdx.x == 0) c->n_groups = t;
-}
-
+// First particle and count of every group.  Each block adds up the counts of
+// the blocks before it (at most n / 4096 words) rather than waiting for a scan
+// of them; a group ends at the next flag, at most 256 positions on.
 __global__ void __launch_bounds__(kFlagThreads)
 bh_flag_write_kernel(const uint8_t* __restrict__ flags, int n, const uint32_t* __restrict__ blk,
-                     int32_t* __restrict__ g_first)
+                     int32_t* __restrict__ g_first, int32_t* __restrict__ g_count, bh_dev_ctrl* c)
 {
-    __shared__ unsigned int ws[kFlagThreads / 32];
+    bh_let_next_start();
+    bh_after_previous(flags, blk, g_first, g_count);
+    constexpr int W = kFlagThreads / 32;
+    __shared__ unsigned int ws[W], wb[W];
+    __shared__ int wfirst[W + 1];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int base = blockIdx.x * kFlagTile + tid * kFlagPer;
-    uint8_t f[kFlagPer];
+    const int base = blockIdx.x * kFlagTile + tid * kFlagPer, end = (blockIdx.x + 1) * kFlagTile;
+    unsigned int before = 0u;
+    for (int i = tid; i < (int)blockIdx.x; i += kFlagThreads) before += blk[i];
+    const uint4 q = *reinterpret_cast<const uint4*>(flags + base);  // 0/1 bytes
+    uint32_t words[4] = {q.x, q.y, q.z, q.w};
     unsigned int s = 0u;
 #pragma unroll
-    for (int i = 0; i < kFlagPer; i++) {
-        f[i] = (base + i < n) ? flags[base + i] : (uint8_t)0;
-        s += f[i];
+    for (int i = 0; i < 4; i++) {
+        const int in = n - base - 4 * i;  // bytes past n may be left from a larger build
+        if (in < 4) words[i] &= in <= 0 ? 0u : (1u << (8 * in)) - 1u;
+        s += __popc(words[i]);
     }
+    int first = n;  // the thread's first flag
+#pragma unroll
+    for (int i = 3; i >= 0; i--)
+        if (words[i]) first = base + 4 * i + ((__ffs(words[i]) - 1) >> 3);
     unsigned int incl = s;
+    int next = first;  // first flag of this or a later lane
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned int t = __shfl_up_sync(BH_FULL_MASK, incl, o);
         if (lane >= o) incl += t;
+        const int u = __shfl_down_sync(BH_FULL_MASK, next, o);
+        if (lane + o < 32) next = min(next, u);
     }
-    if (lane == 31) ws[w] = incl;
+    before = __reduce_add_sync(BH_FULL_MASK, before);
+    // the first flag after the block
+    int after = n;
+    if (end + tid < n && flags[end + tid]) after = end + tid;
+    after = __reduce_min_sync(BH_FULL_MASK, after);
+    if (tid == 0) wfirst[W] = n;
     __syncthreads();
-    unsigned int idx = blk[blockIdx.x] + incl - s;
-    for (int i = 0; i < w; i++) idx += ws[i];
+    if (lane == 31) ws[w] = incl;
+    if (lane == 0) {
+        wb[w] = before;
+        wfirst[w] = next;
+        atomicMin(&wfirst[W], after);
+    }
+    next = __shfl_down_sync(BH_FULL_MASK, next, 1);
+    if (lane == 31) next = n;
+    __syncthreads();
+    unsigned int idx = incl - s;
+    for (int i = 0; i < W; i++) {
+        idx += wb[i];
+        if (i < w) idx += ws[i];
+    }
+    for (int i = w + 1; i <= W; i++) next = min(next, wfirst[i]);
+    if (blockIdx.x == gridDim.x - 1 && tid == kFlagThreads - 1) c->n_groups = idx + s;
+    // the thread's groups, last first: each ends where the one after it begins
+    idx += s;
 #pragma unroll
-    for (int i = 0; i < kFlagPer; i++)
-        if (f[i]) g_first[idx++] = base + i;
-}
-
-__global__ void __launch_bounds__(256) bh_group_count_kernel(const int32_t* __restrict__ g_first,
-                                                             int32_t* __restrict__ g_count, int n,
-                                                             const bh_dev_ctrl* __restrict__ c)
-{
-    const int ng = (int)c->n_groups;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x)
-        g_count[g] = ((g + 1 < ng) ? g_first[g + 1] : n) - g_first[g];
+    for (int i = kFlagPer - 1; i >= 0; i--)
+        if ((words[i >> 2] >> (8 * (i & 3))) & 1u) {
+            idx--;
+            g_first[idx] = base + i;
+            g_count[idx] = next - (base + i);
+            next = base + i;
+        }
 }
 
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
@@ -452,12 +498,10 @@ void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* b
 {
     if (n <= 0) return;
     const int nblk = (n + kFlagTile - 1) / kFlagTile;
-    cudaMemsetAsync(flags, 0, (size_t)nblk * kFlagTile, s);
-    bh_group_mark_kernel<<<grid, 256, 0, s>>>(nd, G, flags, ctrl);
-    bh_flag_count_kernel<<<nblk, kFlagThreads, 0, s>>>(flags, n, blk);
-    bh_flag_scan_kernel<<<1, 1024, 0, s>>>(blk, nblk, ctrl);
-    bh_flag_write_kernel<<<nblk, kFlagThreads, 0, s>>>(flags, n, blk, g_first);
-    bh_group_count_kernel<<<grid, 256, 0, s>>>(g_first, g_count, n, ctrl);
+    // (the flags were cleared by bh_levels_kernel)
+    bh_launch_after(bh_group_mark_kernel, grid, 256, 0, s, nd, G, flags, ctrl);
+    bh_launch_after(bh_flag_count_kernel, nblk, kFlagThreads, 0, s, flags, n, blk);
+    bh_launch_after(bh_flag_write_kernel, nblk, kFlagThreads, 0, s, flags, n, blk, g_first, g_count, ctrl);
 }
 
 // ------------------------------------------------------------ moments
@@ -540,6 +584,8 @@ template <int ORDER>
 __global__ void __launch_bounds__(256) bh_bigleaf_moments_kernel(const float4* __restrict__ pos_s, bh_nodes nd,
                                                                   const bh_dev_ctrl* __restrict__ c)
 {
+    bh_let_next_start();
+    bh_after_previous(pos_s, c);
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     const int nn = (int)c->n_nodes;
@@ -881,6 +927,8 @@ bh_moments_level_kernel(const float4* __restrict__ pos_s, const K* __restrict__ 
                         float theta, int fp64_threshold, int curve, const bh_dev_ctrl* __restrict__ c,
                         const uint32_t* __restrict__ sys, const float4* __restrict__ sys_box)
 {
+    bh_let_next_start();
+    bh_after_previous(pos_s, keys, c, sys, sys_box);
     const int v0 = (int)c->level_offset[lev], v1 = (int)c->level_offset[lev + 1];
     if (c->n_nodes == 0u) return;
     const float4 gbox = make_float4(c->box[0], c->box[1], c->box[2], c->box[3]);
@@ -895,23 +943,23 @@ static void bh_moments_t(const float4* pos_s, const K* keys, const bh_nodes& nd,
                          int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                          const uint32_t* sys, const float4* sys_box)
 {
-    if (order >= 2) bh_bigleaf_moments_kernel<2><<<grid, 256, 0, s>>>(pos_s, nd, ctrl);
-    else bh_bigleaf_moments_kernel<1><<<grid, 256, 0, s>>>(pos_s, nd, ctrl);
+    if (order >= 2) bh_launch_after(bh_bigleaf_moments_kernel<2>, grid, 256, 0, s, pos_s, nd, ctrl);
+    else bh_launch_after(bh_bigleaf_moments_kernel<1>, grid, 256, 0, s, pos_s, nd, ctrl);
     for (int lev = bh_key_traits<K>::kMaxLevel; lev >= 0; lev--) {
         const bool warp = lev <= kWarpMomentLevels;
         if (order >= 2) {
             if (warp)
-                bh_moments_level_kernel<2, K, 32><<<grid, 256, 0, s>>>(pos_s, keys, nd, lev, theta, fp64_threshold,
+                bh_launch_after(bh_moments_level_kernel<2, K, 32>, grid, 256, 0, s, pos_s, keys, nd, lev, theta, fp64_threshold,
                                                                        curve, ctrl, sys, sys_box);
             else
-                bh_moments_level_kernel<2, K, 1><<<grid, 256, 0, s>>>(
+                bh_launch_after(bh_moments_level_kernel<2, K, 1>, grid, 256, 0, s, 
                     pos_s, keys, nd, lev, theta, fp64_threshold, curve, ctrl, sys, sys_box);
         } else {
             if (warp)
-                bh_moments_level_kernel<1, K, 32><<<grid, 256, 0, s>>>(pos_s, keys, nd, lev, theta, fp64_threshold,
+                bh_launch_after(bh_moments_level_kernel<1, K, 32>, grid, 256, 0, s, pos_s, keys, nd, lev, theta, fp64_threshold,
                                                                        curve, ctrl, sys, sys_box);
             else
-                bh_moments_level_kernel<1, K, 1><<<grid, 256, 0, s>>>(
+                bh_launch_after(bh_moments_level_kernel<1, K, 1>, grid, 256, 0, s, 
                     pos_s, keys, nd, lev, theta, fp64_threshold, curve, ctrl, sys, sys_box);
         }
     }

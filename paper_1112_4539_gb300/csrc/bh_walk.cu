@@ -45,6 +45,8 @@ template <int T, int ORDER, bool LEARNED>
 __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
     bh_walk_kernel(WalkParams P)
 {
+    bh_let_next_start();
+    bh_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
@@ -369,6 +371,8 @@ __host__ __device__ constexpr int bh_ws_min_blocks() { return T <= 1 ? 3 : 2; }
 template <int T, int ORDER>
 __global__ void __launch_bounds__(256, bh_ws_min_blocks<T>()) bh_walk_ws_kernel(WalkParams P)
 {
+    bh_let_next_start();
+    bh_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int pair = wib & (kWsPairs - 1);
@@ -683,7 +687,7 @@ static int bh_walk_ws_launch(const WalkParams& P, int sm_count, cudaStream_t s)
         return BH_ERR_CUDA;
     int bps = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, 256, smem) != cudaSuccess || bps < 1) bps = 1;
-    kern<<<sm_count * bps, 256, smem, s>>>(P);
+    bh_launch_after(kern, sm_count * bps, 256, smem, s, P);
     return BH_OK;
 }
 
@@ -758,6 +762,8 @@ struct TmaLanding {
 template <int T, int ORDER>
 __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, false>()) bh_walk_tma_kernel(WalkParams P)
 {
+    bh_let_next_start();
+    bh_after_previous();
     constexpr int RF = bh_wrec_f4(ORDER);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1127,7 +1133,7 @@ static int bh_walk_tma_launch_t(const WalkParams& P, int sm_count, int block_thr
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, block_threads, smem) != cudaSuccess || bps < 1)
             bps = 1;
     }
-    kern<<<sm_count * bps, block_threads, smem, s>>>(P);
+    bh_launch_after(kern, sm_count * bps, block_threads, smem, s, P);
     return BH_OK;
 }
 
@@ -1193,6 +1199,8 @@ void launch_selftest_tma(bh_dev_ctrl* c, cudaStream_t s)
 
 __global__ void bh_walk_reset_kernel(bh_dev_ctrl* c)
 {
+    bh_let_next_start();
+    bh_after_previous();
     c->group_ctr = 0u;
     c->n_pp = 0ull;
     c->n_pc = 0ull;
@@ -1216,7 +1224,7 @@ static int bh_walk_launch_t(const WalkParams& P, int sm_count, int block_threads
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, block_threads, smem) != cudaSuccess || bps < 1)
             bps = 1;
     }
-    kern<<<sm_count * bps, block_threads, smem, s>>>(P);
+    bh_launch_after(kern, sm_count * bps, block_threads, smem, s, P);
     return BH_OK;
 }
 
@@ -1248,7 +1256,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl, int sm_count,
                 int block_threads, int blocks_per_sm, int n, cudaStream_t s, const WalkLearned* learned, int walk_variant)
 {
-    bh_walk_reset_kernel<<<1, 1, 0, s>>>(ctrl);
+    bh_launch_after(bh_walk_reset_kernel, 1, 1, 0, s, ctrl);
     WalkParams P;
     P.pos_s = pos_s;
     P.perm = perm;

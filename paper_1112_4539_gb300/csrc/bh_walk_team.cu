@@ -89,6 +89,8 @@ __host__ __device__ constexpr size_t bh_team_smem_bytes()
 template <int T, int ORDER, int NW>
 __global__ void __launch_bounds__(NW * 32, (T <= 3 ? 16 : 8) / NW) bh_walk_team_kernel(WalkParams P)
 {
+    bh_let_next_start();
+    bh_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // A block's warps sit on the SM's schedulers in turn; the walker, which
     // issues little, is another warp in each of the blocks that share an SM.
@@ -424,7 +426,7 @@ static int bh_team_launch(const WalkParams& P, int n, int sm_count, cudaStream_t
     int bps = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, NW * 32, smem) != cudaSuccess || bps < 1)
         return BH_ERR_CUDA;
-    kern<<<std::min(sm_count * bps, n), NW * 32, smem, s>>>(P);  // at most a group per particle
+    bh_launch_after(kern, std::min(sm_count * bps, n), NW * 32, smem, s, P);  // at most a group per particle
     return BH_OK;
 }
 

@@ -122,16 +122,7 @@ struct PAcc {
     float x, y, z, p, cx, cy, cz, cp;
 };
 
-// 1 / sqrt(a) of the lanes whose bit is set in the masks (as float bits), else
-// 0.  NORMAL: a is known to be no denormal, which saves rsqrtf's scaling.
-template <bool NORMAL>
-__device__ __forceinline__ float bh_rsqrt_of(float a)
-{
-    if (!NORMAL) return rsqrtf(a);
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-    return r;
-}
+// 1 / sqrt(a) of the lanes whose bit is set in the masks (as float bits), else 0.
 template <bool NORMAL>
 __device__ __forceinline__ f2 bh_rsqrt_masked(f2 a, f2 mask, unsigned int bit)
 {

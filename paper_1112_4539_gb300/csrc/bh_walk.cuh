@@ -173,6 +173,15 @@ __device__ __forceinline__ f2 bh_add2(f2 a, f2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ f2 bh_mul2(f2 a, f2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ f2 bh_fma2(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ f2 bh_rsqrt2(f2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+// 1 / sqrt(a).  NORMAL: a is known to be no denormal, which saves rsqrtf's scaling.
+template <bool NORMAL>
+__device__ __forceinline__ float bh_rsqrt_of(float a)
+{
+    if (!NORMAL) return rsqrtf(a);
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 __device__ __forceinline__ f2 bh_lo(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ f2 bh_hi(float4 v) { return make_float2(v.z, v.w); }
 

@@ -1,0 +1,53 @@
+"""Direct sums at the edges of the source tiles and splits against long-double
+sums on the host: both precisions, self terms anywhere, no softening."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _reference(src, tgt, idx, e2):
+    """(sums, sums of magnitudes) in long double; e2[i, j]: squared softening of a pair."""
+    s, t = src.astype(np.longdouble), tgt.astype(np.longdouble)
+    d = s[None, :, :3] - t[:, None, :3]
+    r2 = (d * d).sum(2) + e2
+    m = np.broadcast_to(s[:, 3], r2.shape).copy()
+    for k, j in enumerate(idx):
+        if j >= 0:
+            m[k, j], r2[k, j] = 0, 1
+    w = m / np.sqrt(r2)
+    a = (w / r2)[:, :, None] * d
+    out = np.concatenate([a.sum(1), -w.sum(1)[:, None]], 1)
+    mag = np.concatenate([np.abs(a).sum(1), w.sum(1)[:, None]], 1)
+    return out, mag
+
+
+# of the sum of magnitudes: plain sums of 256 (FP64) or 2 x 128 (FP32) terms of 4 roundings each, compensated across tiles
+TOL = {64: (256 + 8) * 2.0 ** -53, 32: (128 + 8) * 2.0 ** -24}
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("n", [1, 2, 255, 256, 257, 513, 1025, 5000])
+@pytest.mark.parametrize("kind", ["softened", "bare", "symmetrized"])
+def test_tiles(n, precision, kind):
+    import paper_1112_4539_gb300 as bh
+    pos = workloads.plummer(n, seed=n)
+    nt = min(n + 3, 700)
+    tgt = np.concatenate([pos, workloads.plummer(3, seed=99)])[-nt:]
+    idx = np.concatenate([np.arange(n), [-1, -1, -1]])[-nt:]
+    eps = 0.0 if kind == "bare" else 0.01
+    es, et = workloads.softening_lengths(n, 0.01), workloads.softening_lengths(nt, 0.01, seed=5)
+    e2 = (0.5 * (es.astype(np.longdouble) ** 2)[None, :] + 0.5 * (et.astype(np.longdouble) ** 2)[:, None]
+          if kind == "symmetrized" else np.longdouble(eps) ** 2)
+    want, mag = _reference(pos, tgt, idx, e2)
+    d = [torch.from_numpy(a).cuda() for a in (pos, tgt, idx.astype(np.int64), es, et)]
+    out = torch.empty((nt, 4), device="cuda", dtype=torch.float64 if precision == 64 else torch.float32)
+    rc = (bh.direct_force_sym(d[0], d[3], d[1], d[4], d[2], out, precision) if kind == "symmetrized"
+          else bh.direct_force(d[0], d[1], d[2], eps, out, precision))
+    assert rc == 0
+    got = out.cpu().numpy().astype(np.longdouble)
+    assert (np.abs(got - want) <= TOL[precision] * mag + np.longdouble(1e-300)).all()
+

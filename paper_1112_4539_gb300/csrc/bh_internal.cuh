@@ -430,14 +430,14 @@ void launch_softening(const float* eps, const uint32_t* perm, const float4* pos_
 
 int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                const bh_nodes& nd, float4* blo, float4* bhi, int G, const float* h, float h_const, int32_t* count,
-               float* rho, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
+               float* rho, int32_t* heavy, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
 
 // launches per call (deep = 63-bit keys: 8 sort passes, 22 levels)
 inline int launches_build(bool deep) { return deep ? 18 : 14; }  // init, bbox, keys, sort passes, 4 tree, 3 groups
 inline int launches_moments(bool deep) { return (deep ? 22 : 11) + 1; }  // large leaves, one per level
 constexpr int kLaunchesForce = 2;    // counter reset, walk
 constexpr int kLaunchesPWalk = 4;    // parent links, next links, counter reset, walk
-inline int launches_sph(bool deep) { return (deep ? 22 : 11) + 2; }  // node boxes per level, reset, walk
+inline int launches_sph(bool deep) { return (deep ? 22 : 11) + 3; }  // node boxes per level, reset, two walks
 inline int launches_softening(bool deep) { return (deep ? 22 : 11) + 1; }  // gather, one per level
 
 }  // namespace bh

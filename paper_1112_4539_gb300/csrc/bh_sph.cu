@@ -8,11 +8,18 @@
 // particles: a node is skipped when its particles' bounding box lies farther
 // than the group's largest radius from the group's bounding box (with a
 // 1e-5 relative allowance, so FP32 rounding of the box gap can never skip a
-// neighbour), a leaf contributes all its particles as candidates when its
-// box is also within reach of at least one target of the warp (each with its
-// own radius), other nodes are opened.  Candidates go through a 64-entry
-// ring in shared memory and are tested 32 at a time against each lane's T
-// targets.
+// neighbour), a leaf is taken when its box is also within reach of at least one
+// target of the warp (each with its own radius), other nodes are opened.  The
+// particles of a taken leaf that lie within the largest radius of the group's
+// box become candidates; they go through a 64-entry ring in shared memory, as
+// pairs, and are tested 32 at a time against each lane's T targets.
+//
+// Bound by instruction issue: about 6 candidates are tested per neighbour found,
+// and some lane has a hit at nearly every one.  Against the form that took
+// every particle of a leaf, one at a time, with a test for the target itself
+// (GB300, build and search, Plummer, 64 neighbours): 2^20, G = 32 1.42 -> 1.08 ms
+// (510 -> 395 M candidate pairs), 2^20, G = 64 1.61 -> 1.24 ms, 2^24, G = 32
+// 28.1 -> 15.8 ms (21.9 -> 8.1 G pairs).
 //
 // Pair rule (identical to the oracle's): d = x_j - x_i per axis in FP32,
 // r2 = fma(dz, dz, fma(dy, dy, dx * dx)), j != i is a neighbour iff
@@ -21,23 +28,20 @@
 // Lattanzio 1985), FP32.
 #include <algorithm>
 
-#include "bh_internal.cuh"
+#include "bh_walk.cuh"
 
 namespace bh {
 
-#ifndef BH_SPH_LEAF_FILTER
-#define BH_SPH_LEAF_FILTER 1
-#endif
-constexpr int kSphStackCap = 704;   // ranges of <= 8 siblings; same bound as the gravity walk
-constexpr int kSphRing = 64;
+constexpr int kSphStackCap = kStackCap;  // ranges of <= 8 siblings; same bound as the gravity walk
+constexpr int kSphRing = 64;             // candidates per ring (two tiles of 32)
 
 // ------------------------------------------------------------ node boxes
 // Tight bounding box of every node's particles, bottom-up by level: a leaf
 // scans its particles, an internal node combines its children (one level
 // deeper, already done).  Min/max are exact.
-__global__ void bh_node_box_kernel(const float4* __restrict__ pos_s, const int4* __restrict__ rec,
-                                   float4* __restrict__ lo, float4* __restrict__ hi, int lev,
-                                   const bh_dev_ctrl* __restrict__ c)
+__global__ void __launch_bounds__(256)
+bh_node_box_kernel(const float4* __restrict__ pos_s, const int4* __restrict__ rec, float4* __restrict__ lo,
+                   float4* __restrict__ hi, int lev, const bh_dev_ctrl* __restrict__ c)
 {
     bh_let_next_start();
     bh_after_previous(pos_s, rec, lo, hi, c);
@@ -45,17 +49,32 @@ __global__ void bh_node_box_kernel(const float4* __restrict__ pos_s, const int4*
     for (int v = v0 + blockIdx.x * blockDim.x + threadIdx.x; v < v1; v += gridDim.x * blockDim.x) {
         const int4 r = rec[v];
         float4 a = make_float4(INFINITY, INFINITY, INFINITY, 0.f), b = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.f);
+        // loads in batches: the pass waits for little else
         if (r.z < 0) {
-            for (int k = r.x; k < r.x + r.y; k++) {
-                const float4 p = pos_s[k];
-                a.x = fminf(a.x, p.x); a.y = fminf(a.y, p.y); a.z = fminf(a.z, p.z);
-                b.x = fmaxf(b.x, p.x); b.y = fmaxf(b.y, p.y); b.z = fmaxf(b.z, p.z);
+            for (int k = 0; k < r.y; k += 8) {
+                float4 p[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++) p[u] = pos_s[r.x + min(k + u, r.y - 1)];  // (repeats change no bound)
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    a.x = fminf(a.x, p[u].x); a.y = fminf(a.y, p[u].y); a.z = fminf(a.z, p[u].z);
+                    b.x = fmaxf(b.x, p[u].x); b.y = fmaxf(b.y, p[u].y); b.z = fmaxf(b.z, p[u].z);
+                }
             }
         } else {
-            for (int k = r.z; k < r.z + r.w; k++) {
-                const float4 l = lo[k], h = hi[k];
-                a.x = fminf(a.x, l.x); a.y = fminf(a.y, l.y); a.z = fminf(a.z, l.z);
-                b.x = fmaxf(b.x, h.x); b.y = fmaxf(b.y, h.y); b.z = fmaxf(b.z, h.z);
+#pragma unroll
+            for (int k = 0; k < 8; k += 4) {
+                float4 l[4], h[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    l[u] = lo[r.z + min(k + u, r.w - 1)];
+                    h[u] = hi[r.z + min(k + u, r.w - 1)];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    a.x = fminf(a.x, l[u].x); a.y = fminf(a.y, l[u].y); a.z = fminf(a.z, l[u].z);
+                    b.x = fmaxf(b.x, h[u].x); b.y = fmaxf(b.y, h[u].y); b.z = fmaxf(b.z, h[u].z);
+                }
             }
         }
         lo[v] = a;
@@ -66,10 +85,9 @@ __global__ void bh_node_box_kernel(const float4* __restrict__ pos_s, const int4*
 // ------------------------------------------------------------ walk
 struct SphSmem {
     uint32_t stack[kSphStackCap];
-    uint32_t staging[32];
-    int2 leafq[64];
-    float4 ring[kSphRing];   // candidate particles (x, y, z, m)
-    int ridx[kSphRing];      // their Morton positions (self test)
+    int2 leafq[32];
+    float4 blo[32], bhi[32];                      // boxes of the pop's near leaves
+    float4 ra[kSphRing / 2], rb[kSphRing / 2];    // candidates as pairs: (x, x', y, y') (z, z', m, m')
 };
 
 struct SphParams {
@@ -85,6 +103,7 @@ struct SphParams {
     int32_t* count;      // caller order (nullptr: not written)
     float* rho;          // caller order (nullptr: not written)
     bh_dev_ctrl* ctrl;
+    int32_t* heavy;      // groups left to the second launch (tile_ctr[0] of them)
 };
 
 // cubic spline with support h (normalised to unit integral), FP32
@@ -96,57 +115,94 @@ __device__ __forceinline__ float bh_w3(float r, float hinv, float c)
     return c * (q <= 0.5f ? inner : (q <= 1.0f ? 2.0f * u * u * u : 0.0f));
 }
 
+// np pairs of candidates against the lane's targets; (nx, ny, nz): minus the
+// target, held twice.  The target itself is among the candidates once, at r2 =
+// 0 (the caller starts its count at -1).
 template <int T>
-__device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ src, const int* __restrict__ sidx, int gb,
-                                            const float (&xi)[T], const float (&yi)[T], const float (&zi)[T],
-                                            const float (&h2)[T], const float (&hinv)[T], const float (&cw)[T],
-                                            int tn, int (&cnt)[T], float (&rho)[T])
+__device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const float4* __restrict__ rb, int np,
+                                            const f2 (&nx)[T], const f2 (&ny)[T], const f2 (&nz)[T],
+                                            const float (&h2)[T], const float (&hinv)[T], const float (&cw)[T], int tn,
+                                            int (&cnt)[T], float (&rho)[T])
 {
-    const int lane = threadIdx.x & 31;
-    for (int j = 0; j < 32; j++) {
-        const float4 s = src[j];
-        const int js = sidx[j];
+#pragma unroll 4
+    for (int j = 0; j < np; j++) {
+        const float4 sa = ra[j], sb = rb[j];
 #pragma unroll
         for (int t = 0; t < T; t++) {
             if (t < tn) {
-                const float dx = __fsub_rn(s.x, xi[t]), dy = __fsub_rn(s.y, yi[t]), dz = __fsub_rn(s.z, zi[t]);
-                const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-                const bool self = js == gb + t * 32 + lane;
-                if (r2 < h2[t] || self) {
-                    cnt[t] += self ? 0 : 1;
-                    rho[t] = fmaf(s.w, bh_w3(sqrtf(r2), hinv[t], cw[t]), rho[t]);
+                const f2 dx = bh_add2(bh_lo(sa), nx[t]), dy = bh_add2(bh_hi(sa), ny[t]), dz = bh_add2(bh_lo(sb), nz[t]);
+                const f2 r2 = bh_fma2(dz, dz, bh_fma2(dy, dy, bh_mul2(dx, dx)));
+                if (r2.x < h2[t]) {
+                    cnt[t]++;
+                    rho[t] = fmaf(sb.z, bh_w3(sqrtf(r2.x), hinv[t], cw[t]), rho[t]);
+                }
+                if (r2.y < h2[t]) {
+                    cnt[t]++;
+                    rho[t] = fmaf(sb.w, bh_w3(sqrtf(r2.y), hinv[t], cw[t]), rho[t]);
                 }
             }
         }
     }
 }
 
+// NW = 1: a warp per group, which gives up a group after kSphHeavy candidates or
+// kSphPops batches of nodes and lists it.  NW > 1: a block of NW warps per
+// listed group, which share its subtrees; their counts and densities are added
+// in warp order.  A group's work varies with its radii (in a Plummer sphere's
+// outskirts the radius that holds 64 neighbours reaches into the core), and the
+// few long ones were the whole tail of the launch.
+//
+// GB300, build and search, a warp per group throughout -> this (the same counts):
+// Plummer 131072, G = 32 1.56 -> 0.77 ms, 4000 particles 580 -> 477 us, 2^20
+// unchanged.  Limits of 32 / 64 / 128 batches: 2^20 1.17 / 1.09 / 1.09 ms, 131072
+// 0.72 / 0.77 / 0.90 ms; of 512 / 1024 / 2048 candidates at 2^20 1.17 / 1.10 / 1.10.
+constexpr int kSphHeavy = 1024;
+constexpr int kSphPops = 64;
+constexpr int kSphSplit = 4;  // the level whose subtrees are shared out
 template <int T>
-__global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
+constexpr int bh_sph_team() { return T <= 3 ? 8 : 4; }  // (shared memory)
+template <int T, int NW>
+__global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphParams P)
 {
     bh_let_next_start();
     bh_after_previous();
-    __shared__ SphSmem smem[4];
+    __shared__ SphSmem smem[NW == 1 ? 4 : NW];
+    __shared__ int s_group;
+    __shared__ float s_rho[NW == 1 ? 1 : NW * T * 32];
+    __shared__ int s_cnt[NW == 1 ? 1 : NW * T * 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     SphSmem& S = smem[wib];
     const unsigned int lt = bh_lanemask_lt();
     bh_dev_ctrl* ctrl = P.ctrl;
     const int ng = (int)ctrl->n_groups;
     const int n_roots = (int)ctrl->level_offset[1];
+    const int split = (int)ctrl->level_offset[kSphSplit], below = (int)ctrl->level_offset[kSphSplit + 1];
     unsigned long long tested = 0ull;
 
     for (;;) {
         int g = 0;
-        if (lane == 0) g = (int)atomicAdd(&ctrl->group_ctr, 1u);
-        g = __shfl_sync(BH_FULL_MASK, g, 0);
-        if (g >= ng) break;
-        int ab = 0;
-        if (lane == 0) ab = (int)*(volatile unsigned int*)&ctrl->abort;
-        if (__shfl_sync(BH_FULL_MASK, ab, 0)) break;
+        if (NW == 1) {
+            if (lane == 0) {
+                g = (int)atomicAdd(&ctrl->group_ctr, 1u);
+                if (*(volatile unsigned int*)&ctrl->abort) g = ng;
+            }
+            g = __shfl_sync(BH_FULL_MASK, g, 0);
+            if (g >= ng) break;
+        } else {
+            __syncthreads();  // the last group's sums have been read
+            if (threadIdx.x == 0) {
+                const unsigned int k = atomicAdd(&ctrl->tile_ctr[1], 1u);
+                s_group = (k < ctrl->tile_ctr[0] && !*(volatile unsigned int*)&ctrl->abort) ? P.heavy[k] : -1;
+            }
+            __syncthreads();
+            g = s_group;
+            if (g < 0) break;
+        }
         const int gb = P.g_first[g], gc = P.g_count[g];
         const int tn = (gc + 31) >> 5;
 
         float xi[T], yi[T], zi[T], h2[T], hinv[T], cw[T], rho[T];
+        f2 nx[T], ny[T], nz[T];
         int cnt[T];
         float bx0 = INFINITY, by0 = INFINITY, bz0 = INFINITY, bx1 = -INFINITY, by1 = -INFINITY, bz1 = -INFINITY;
         float hmax = 0.0f;
@@ -168,8 +224,11 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
             h2[t] = __fmul_rn(h, h);
             hinv[t] = 1.0f / h;
             cw[t] = 8.0f / (3.14159265358979f * h * h * h);
-            cnt[t] = 0;
-            rho[t] = 0.0f;
+            nx[t] = make_float2(-q.x, -q.x); ny[t] = make_float2(-q.y, -q.y); nz[t] = make_float2(-q.z, -q.z);
+            // the target's own pair has r2 = 0, below h^2 unless that underflows
+            const bool own = h2[t] > 0.0f, first = NW == 1 || wib == 0;
+            cnt[t] = own && first ? -1 : 0;
+            rho[t] = own || !first ? 0.0f : q.w * bh_w3(0.0f, hinv[t], cw[t]);
         }
         if (__any_sync(BH_FULL_MASK, bad)) {
             if (lane == 0) bh_set_error(ctrl, BH_ERR_NONFINITE);
@@ -186,12 +245,10 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
             hmax = fmaxf(hmax, __shfl_xor_sync(BH_FULL_MASK, hmax, o));
         }
         const float reach2 = hmax * hmax * (1.0f + 1e-5f);
-#if BH_SPH_LEAF_FILTER
         // each target's own reach for the leaf filter (-1: no target in the slot)
         float reach_t[T];
 #pragma unroll
         for (int t = 0; t < T; t++) reach_t[t] = (t * 32 + lane < gc) ? h2[t] * (1.0f + 1e-5f) : -1.0f;
-#endif
 
         // root of the group's system
         int root = 0;
@@ -200,32 +257,19 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
             if (P.rec[mid].x <= gb) root = mid;
             else hi = mid;
         }
-        int sp = 1, ring_head = 0, ring_cnt = 0;
+        int sp = 1, ring_head = 0, ring_cnt = 0, pops = 0, taken = 0;
         if (lane == 0) S.stack[0] = (uint32_t)root << 3;
         __syncwarp();
-        bool overflow = false;
+        bool overflow = false, heavy = false;
         while (sp > 0) {
-            // pop the top 32 nodes
-            int c = 0;
-            uint32_t e = 0u;
-            if (lane < sp) {
-                e = S.stack[sp - 1 - lane];
-                c = (int)(e & 7u) + 1;
+            if (NW == 1 && (taken >= kSphHeavy || pops++ >= kSphPops)) {
+                heavy = true;
+                break;
             }
-            const int incl = bh_warp_incl_scan(c);
-            const int excl = incl - c;
-            const int take = max(0, min(c, 32 - excl));
-            const int st = (int)(e >> 3);
-            for (int t = 0; t < take; t++) S.staging[excl + t] = (uint32_t)(st + t);
-            const bool full = (lane < sp) && (take == c);
-            const int nfull = __popc(__ballot_sync(BH_FULL_MASK, full));
-            const int npop = min(__shfl_sync(BH_FULL_MASK, incl, 31), 32);
-            __syncwarp();
-            if (lane == nfull && lane < sp && take > 0)
-                S.stack[sp - 1 - lane] = ((uint32_t)(st + take) << 3) | (uint32_t)(c - take - 1);
-            sp -= nfull;
+            // pop the top 32 nodes
+            int v, row;
+            const int npop = bh_pop_nodes(S.stack, sp, lt, v, row);
             const bool has = lane < npop;
-            const int v = has ? (int)S.staging[lane] : 0;
             __syncwarp();
 
             // distance_test: the node's box against the group's box
@@ -241,32 +285,36 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
                 const float gz = fmaxf(fmaxf(a.z - bz1, bz0 - b.z), 0.0f);
                 near = gx * gx + gy * gy + gz * gz <= reach2;
             }
+            // a block's warps walk the top of the tree alike and share out its
+            // leaves and the subtrees from level kSphSplit down by node index
+            if (NW > 1 && v < below && (v >= split || r.z < 0)) near = near && v % NW == wib;
             bool leaf = near && r.z < 0;
             const bool opn = near && r.z >= 0;
-#if BH_SPH_LEAF_FILTER
             // per-target filter: a leaf near the group's box is kept only when
             // its box lies within reach of at least one target of the warp
             {
-                unsigned int lm0 = __ballot_sync(BH_FULL_MASK, leaf), keep = 0u;
-                while (lm0) {
-                    const int q = __ffs(lm0) - 1;
-                    lm0 &= lm0 - 1u;
-                    const float lx0 = __shfl_sync(BH_FULL_MASK, a.x, q), ly0 = __shfl_sync(BH_FULL_MASK, a.y, q);
-                    const float lz0 = __shfl_sync(BH_FULL_MASK, a.z, q), lx1 = __shfl_sync(BH_FULL_MASK, b.x, q);
-                    const float ly1 = __shfl_sync(BH_FULL_MASK, b.y, q), lz1 = __shfl_sync(BH_FULL_MASK, b.z, q);
+                const unsigned int lm0 = __ballot_sync(BH_FULL_MASK, leaf);
+                const int at = __popc(lm0 & lt), nl = __popc(lm0);
+                if (leaf) {
+                    S.blo[at] = a;
+                    S.bhi[at] = b;
+                }
+                __syncwarp();
+                unsigned int keep = 0u;  // by place in the list
+                for (int q = 0; q < nl; q++) {
+                    const float4 l = S.blo[q], u = S.bhi[q];
                     bool hit = false;
 #pragma unroll
                     for (int t = 0; t < T; t++) {
-                        const float dx = fmaxf(fmaxf(lx0 - xi[t], xi[t] - lx1), 0.0f);
-                        const float dy = fmaxf(fmaxf(ly0 - yi[t], yi[t] - ly1), 0.0f);
-                        const float dz = fmaxf(fmaxf(lz0 - zi[t], zi[t] - lz1), 0.0f);
+                        const float dx = fmaxf(fmaxf(l.x - xi[t], xi[t] - u.x), 0.0f);
+                        const float dy = fmaxf(fmaxf(l.y - yi[t], yi[t] - u.y), 0.0f);
+                        const float dz = fmaxf(fmaxf(l.z - zi[t], zi[t] - u.z), 0.0f);
                         hit = hit || (dx * dx + dy * dy + dz * dz <= reach_t[t]);
                     }
                     if (__any_sync(BH_FULL_MASK, hit)) keep |= 1u << q;
                 }
-                leaf = leaf && ((keep >> lane) & 1u);
+                leaf = leaf && ((keep >> at) & 1u);
             }
-#endif
             const unsigned int om = __ballot_sync(BH_FULL_MASK, opn);
             if (sp + __popc(om) > kSphStackCap) {
                 overflow = true;
@@ -283,39 +331,36 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
             int lq_pos = 0;
             for (;;) {
                 if (ring_cnt >= 32) {
-                    bh_sph_tile<T>(S.ring + ring_head, S.ridx + ring_head, gb, xi, yi, zi, h2, hinv, cw, tn, cnt,
-                                   rho);
-                    tested += 32ull * (unsigned long long)gc;
+                    bh_sph_tile<T>(S.ra + (ring_head >> 1), S.rb + (ring_head >> 1), 16, nx, ny, nz, h2, hinv, cw, tn,
+                                   cnt, rho);
+                    taken += 32;
                     ring_head ^= 32;
                     ring_cnt -= 32;
                     __syncwarp();
                     continue;
                 }
                 if (lq_pos >= lq_n) break;
-                int c2 = 0;
-                int2 q = make_int2(0, 0);
-                if (lq_pos + lane < lq_n) {
-                    q = S.leafq[lq_pos + lane];
-                    c2 = q.y;
-                }
-                const int inc2 = bh_warp_incl_scan(c2);
-                const int ex2 = inc2 - c2;
-                const int take2 = max(0, min(c2, 32 - ex2));
-                for (int t = 0; t < take2; t++) S.staging[ex2 + t] = (uint32_t)(q.x + t);
-                const bool full2 = (lq_pos + lane < lq_n) && (take2 == c2);
-                const int nf2 = __popc(__ballot_sync(BH_FULL_MASK, full2));
-                const int nfill = min(__shfl_sync(BH_FULL_MASK, inc2, 31), 32);
-                __syncwarp();
-                if (lane == nf2 && lq_pos + lane < lq_n && take2 > 0)
-                    S.leafq[lq_pos + lane] = make_int2(q.x + take2, c2 - take2);
-                lq_pos += nf2;
+                // candidates: the leaves' particles within the largest radius of the group's box
+                int k;
+                const int nfill = bh_take_particles(S.leafq, lq_pos, lq_n, lt, k, row);
+                bool in = false;
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (lane < nfill) {
-                    const int k = (int)S.staging[lane];
-                    const int slot = (ring_head + ring_cnt + lane) & (kSphRing - 1);
-                    S.ring[slot] = P.pos_s[k];
-                    S.ridx[slot] = k;
+                    p = P.pos_s[k];
+                    const float gx = fmaxf(fmaxf(p.x - bx1, bx0 - p.x), 0.0f);
+                    const float gy = fmaxf(fmaxf(p.y - by1, by0 - p.y), 0.0f);
+                    const float gz = fmaxf(fmaxf(p.z - bz1, bz0 - p.z), 0.0f);
+                    in = gx * gx + gy * gy + gz * gz <= reach2;
                 }
-                ring_cnt += nfill;
+                const unsigned int im = __ballot_sync(BH_FULL_MASK, in);
+                if (in) {
+                    const int slot = (ring_head + ring_cnt + __popc(im & lt)) & (kSphRing - 1);
+                    float* fa = reinterpret_cast<float*>(&S.ra[slot >> 1]) + (slot & 1);
+                    float* fb = reinterpret_cast<float*>(&S.rb[slot >> 1]) + (slot & 1);
+                    fa[0] = p.x; fa[2] = p.y;
+                    fb[0] = p.z; fb[2] = p.w;
+                }
+                ring_cnt += __popc(im);
                 __syncwarp();
             }
         }
@@ -323,17 +368,49 @@ __global__ void __launch_bounds__(128) bh_sph_kernel(SphParams P)
             if (lane == 0) bh_set_error(ctrl, BH_ERR_CAPACITY);
             break;
         }
+        if (heavy) {
+            if (lane == 0) P.heavy[atomicAdd(&ctrl->tile_ctr[0], 1u)] = g;
+            continue;
+        }
         if (ring_cnt > 0) {
-            // pad with far, massless candidates that match no index
-            if (lane >= ring_cnt) {
-                S.ring[ring_head + lane] = make_float4(INFINITY, INFINITY, INFINITY, 0.0f);
-                S.ridx[ring_head + lane] = -1;
+            // an odd last candidate gets a far one beside it, which is nobody's neighbour
+            if (lane == 0 && (ring_cnt & 1)) {
+                const int slot = ring_head + ring_cnt;
+                float* fa = reinterpret_cast<float*>(&S.ra[slot >> 1]) + 1;
+                float* fb = reinterpret_cast<float*>(&S.rb[slot >> 1]) + 1;
+                fa[0] = fa[2] = fb[0] = INFINITY;
+                fb[2] = 0.0f;
             }
             __syncwarp();
-            bh_sph_tile<T>(S.ring + ring_head, S.ridx + ring_head, gb, xi, yi, zi, h2, hinv, cw, tn, cnt, rho);
-            tested += (unsigned long long)ring_cnt * (unsigned long long)gc;
+            bh_sph_tile<T>(S.ra + (ring_head >> 1), S.rb + (ring_head >> 1), (ring_cnt + 1) >> 1, nx, ny, nz, h2, hinv,
+                           cw, tn, cnt, rho);
+            taken += ring_cnt;
         }
+        tested += (unsigned long long)taken * (unsigned long long)gc;
         __syncwarp();
+        if (NW > 1) {
+#pragma unroll
+            for (int t = 0; t < T; t++) {
+                s_cnt[(wib * T + t) * 32 + lane] = cnt[t];
+                s_rho[(wib * T + t) * 32 + lane] = rho[t];
+            }
+            __syncthreads();
+            for (int t = wib; t < T; t += NW) {
+                int c = 0;
+                float d = 0.0f;
+                for (int w = 0; w < NW; w++) {
+                    c += s_cnt[(w * T + t) * 32 + lane];
+                    d += s_rho[(w * T + t) * 32 + lane];
+                }
+                const int o = t * 32 + lane;
+                if (o < gc) {
+                    const uint32_t dst = P.perm[gb + o];
+                    if (P.count) P.count[dst] = c;
+                    if (P.rho) P.rho[dst] = d;
+                }
+            }
+            continue;
+        }
 #pragma unroll
         for (int t = 0; t < T; t++) {
             const int o = t * 32 + lane;
@@ -355,26 +432,35 @@ __global__ void bh_sph_reset_kernel(bh_dev_ctrl* c)
     bh_let_next_start();
     bh_after_previous();
     c->group_ctr = 0u;
+    c->tile_ctr[0] = 0u;  // groups listed as heavy (the sort's tickets are free after the build)
+    c->tile_ctr[1] = 0u;  // and taken
     c->n_pp = 0ull;
     c->n_pc = 0ull;
 }
 
 // persistent grid: as many blocks per SM as the registers and shared memory allow
+template <int T, int NW>
+static void bh_sph_launch_nw(const SphParams& P, int sm_count, cudaStream_t s)
+{
+    constexpr int threads = NW == 1 ? 128 : NW * 32;
+    int bps = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, bh_sph_kernel<T, NW>, threads, 0) != cudaSuccess || bps < 1) {
+        cudaGetLastError();
+        bps = 1;
+    }
+    bh_launch_after(bh_sph_kernel<T, NW>, sm_count * bps, threads, 0, s, P);
+}
 template <int T>
 static int bh_sph_launch(const SphParams& P, int sm_count, cudaStream_t s)
 {
-    int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, bh_sph_kernel<T>, 128, 0) != cudaSuccess || bps < 1) {
-        cudaGetLastError();
-        bps = 4;
-    }
-    bh_launch_after(bh_sph_kernel<T>, sm_count * bps, 128, 0, s, P);
+    bh_sph_launch_nw<T, 1>(P, sm_count, s);
+    bh_sph_launch_nw<T, bh_sph_team<T>()>(P, sm_count, s);
     return BH_OK;
 }
 
 int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                const bh_nodes& nd, float4* blo, float4* bhi, int G, const float* h, float h_const, int32_t* count,
-               float* rho, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s)
+               float* rho, int32_t* heavy, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s)
 {
     for (int lev = max_level; lev >= 0; lev--)
         bh_launch_after(bh_node_box_kernel, grid, 256, 0, s, pos_s, nd.rec, blo, bhi, lev, ctrl);
@@ -392,6 +478,7 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
     P.count = count;
     P.rho = rho;
     P.ctrl = ctrl;
+    P.heavy = heavy;
     const int T = G <= 32 ? 1 : G <= 64 ? 2 : G <= 96 ? 3 : G <= 128 ? 4 : 8;
     switch (T) {
         case 1: return bh_sph_launch<1>(P, sm_count, s);

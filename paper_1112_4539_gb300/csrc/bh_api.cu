@@ -30,7 +30,8 @@ struct bh_ctx {
     bh_dev_ctrl* ctrl = nullptr;
     bh_dev_ctrl* host_ctrl = nullptr;  // pinned staging for read-back
     float4* pos_s = nullptr;
-    void *keys = nullptr, *keys_alt = nullptr;   // uint32_t[n] or, deep, uint64_t[n]
+    void *keys = nullptr, *keys_alt = nullptr;   // uint32_t[n] or, deep, uint64_t[n]; after the sort keys_alt
+                                                 // holds the groups by falling cost
     uint32_t *vals = nullptr, *vals_alt = nullptr;
     unsigned long long* lookback = nullptr;
     uint16_t* dl = nullptr;
@@ -303,8 +304,8 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
                         x->deep, s);
         bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap,
                         x->ctrl, grid_for(x), s);
-        bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, x->ctrl,
-                          grid_for(x), s);
+        bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count,
+                          (int32_t*)x->keys_alt, x->ctrl, grid_for(x), s);
         x->launches += bh::launches_build(x->deep) - 1;
     }
     x->launches += 1;
@@ -376,8 +377,8 @@ int tree_force(bh_ctx* x, float eps, float* d_acc_pot, void* stream)
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
     bh::WalkLearned wl{x->mfeat, x->mlp, x->theta};
-    int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, x->nd, x->cfg.order, x->cfg.group_size,
-                             eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
+    int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
+                             x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
                              x->cfg.blocks_per_sm, (int)x->n, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     x->launches += bh::kLaunchesForce;
@@ -745,15 +746,17 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
                           x->pos_s, x->sys_of, x->sys_box, x->cfg.curve, x->deep, x->ctrl, s);
     bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap, x->ctrl,
                     grid_for(x), s, x->sys_of, x->sys_off);
-    bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, x->ctrl, grid_for(x), s);
+    bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, (int32_t*)x->keys_alt,
+                      x->ctrl, grid_for(x), s);
     bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
                        x->cfg.curve, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
-    int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, x->nd, x->cfg.order, x->cfg.group_size, eps,
-                             (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
+    int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
+                             x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count,
+                             x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
-    // init, batch sort, 4 tree, 3 groups, moments per level, 2 walk
-    x->launches += 2 + 4 + 3 + bh::launches_moments(x->deep) + bh::kLaunchesForce;
+    // init, batch sort, 4 tree, 4 groups, moments per level, 2 walk
+    x->launches += 2 + 4 + 4 + bh::launches_moments(x->deep) + bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
     x->theta = theta;

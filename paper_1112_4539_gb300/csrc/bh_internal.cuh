@@ -48,6 +48,8 @@ struct bh_dev_ctrl {
     unsigned int build_seq;      // builds since the block was zeroed (never reset): the sort
                                  // passes of build b use look-back epochs 8 b + 1 .. 8 b + 8
     unsigned int scan_done;      // level-scan blocks finished (the last one writes the offsets)
+    unsigned int cost_count[16]; // groups of each cost class (bh_group_order_kernel)
+    unsigned int cost_taken[16];
     unsigned int pad[6];
 };
 
@@ -381,8 +383,9 @@ void launch_sort(void* keys, void* keys_alt, uint32_t* vals, uint32_t* vals_alt,
 void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, uint8_t* flags,
                  const bh_nodes& nd, int64_t node_cap, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                  const uint32_t* sys = nullptr, const int32_t* sys_off = nullptr);
+// g_order (n words): the groups by falling cost
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
-                   int32_t* g_count, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);
+                   int32_t* g_count, int32_t* g_order, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);
 void launch_moments(const float4* pos_s, const void* keys, bool deep, const bh_nodes& nd, int order,
                     float theta, int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                     const uint32_t* sys = nullptr, const float4* sys_box = nullptr);
@@ -402,6 +405,7 @@ struct WalkLearned {
     float theta_guard;
 };
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
+                const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl,
                 int sm_count, int block_threads, int blocks_per_sm, int n, cudaStream_t s,
                 const WalkLearned* learned = nullptr, int walk_variant = 0);
@@ -433,7 +437,7 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
                float* rho, int32_t* heavy, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
 
 // launches per call (deep = 63-bit keys: 8 sort passes, 22 levels)
-inline int launches_build(bool deep) { return deep ? 18 : 14; }  // init, bbox, keys, sort passes, 4 tree, 3 groups
+inline int launches_build(bool deep) { return deep ? 19 : 15; }  // init, bbox, keys, sort passes, 4 tree, 4 groups
 inline int launches_moments(bool deep) { return (deep ? 22 : 11) + 1; }  // large leaves, one per level
 constexpr int kLaunchesForce = 2;    // counter reset, walk
 constexpr int kLaunchesPWalk = 4;    // parent links, next links, counter reset, walk

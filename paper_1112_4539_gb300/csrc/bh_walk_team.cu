@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(NW * 32, (T <= 3 ? 16 : 8) / NW) bh_walk_team_
             if (next < ng) next = (int)atomicAdd(&ctrl->group_ctr, 1u);
         }
         __syncthreads();
-        const int g = S.group;
-        if (g < 0) break;
+        if (S.group < 0) break;
+        const int g = P.g_order[S.group];
         const int gb = P.g_first[g], gc = P.g_count[g], ge = gb + gc;
         Layout L;
         {

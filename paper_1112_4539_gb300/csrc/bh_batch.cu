@@ -127,8 +127,8 @@ bh_batch_sort_kernel(const float4* __restrict__ pos, const int32_t* __restrict__
                 const bool ok = p < e;
                 key[k] = ok ? sk[p] : (K)0;
                 val[k] = ok ? sv[p] : 0u;
-                const unsigned int d = ok ? ((unsigned int)(key[k] >> shift) & 255u) : 256u;
-                const unsigned int peers = __match_any_sync(BH_FULL_MASK, d);
+                const unsigned int d = (unsigned int)(key[k] >> shift) & 255u;
+                const unsigned int peers = bh_match_digit(d, ok);
                 unsigned int prior = 0u;
                 if (ok) prior = whist[w][d];
                 __syncwarp();

@@ -309,8 +309,7 @@ bh_onesweep_kernel(const K* __restrict__ kin, const uint32_t* __restrict__ vin, 
 #pragma unroll
     for (int k = 0; k < ITEMS; k++) {
         const bool ok = base + w * (32 * ITEMS) + k * 32 + lane < n;
-        const unsigned int d = ok ? ((unsigned int)(key[k] >> shift) & 255u) : 256u;
-        rank[k] = __match_any_sync(BH_FULL_MASK, d);
+        rank[k] = bh_match_digit((unsigned int)(key[k] >> shift) & 255u, ok);
     }
 #pragma unroll
     for (int k = 0; k < ITEMS; k++) {

@@ -296,8 +296,16 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
     cudaStream_t s = (cudaStream_t)stream;
     const int N = (int)n;
     const float4* pos = (const float4*)d_pos_mass;
-    bh::launch_init(x->ctrl, s);
-    if (N > 0) {
+    if (N > 0 && bh::bh_small_set(N, x->deep)) {
+        if (!bh::launch_small_build(pos, N, x->cfg.leaf_size, x->cfg.group_size, x->cfg.curve, x->deep, x->nd,
+                                    x->node_cap, x->keys, x->vals, x->pos_s, x->g_first, x->g_count, x->ctrl, s)) {
+            cudaGetLastError();
+            return BH_ERR_CUDA;
+        }
+    } else {
+        bh::launch_init(x->ctrl, s);
+    }
+    if (N > 0 && !bh::bh_small_set(N, x->deep)) {
         bh::launch_bbox(pos, N, x->ctrl, grid_for(x), s);
         bh::launch_keys(pos, N, x->ctrl, x->keys, x->cfg.curve, x->deep, grid_for(x), s);
         bh::launch_sort(x->keys, x->keys_alt, x->vals, x->vals_alt, pos, x->pos_s, N, x->lookback, x->ctrl,
@@ -306,7 +314,7 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
                         x->ctrl, grid_for(x), s);
         bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count,
                           (int32_t*)x->keys_alt, x->ctrl, grid_for(x), s);
-        x->launches += bh::launches_build(x->deep) - 1;
+        x->launches += bh::launches_build(x->deep) - (bh::bh_groups_ordered(N, x->cfg.group_size) ? 1 : 2);
     }
     x->launches += 1;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
@@ -755,8 +763,8 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
                              x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
-    // init, batch sort, 4 tree, 4 groups, moments per level, 2 walk
-    x->launches += 2 + 4 + 4 + bh::launches_moments(x->deep) + bh::kLaunchesForce;
+    // init, batch sort, 4 tree, 3 or 4 groups, moments per level, 2 walk
+    x->launches += 2 + 4 + (bh::bh_groups_ordered(N, x->cfg.group_size) ? 4 : 3) + bh::launches_moments(x->deep) + bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
     x->theta = theta;

@@ -12,6 +12,7 @@
 //     so the children of a node are contiguous.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -403,6 +404,15 @@ void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* b
 void launch_moments(const float4* pos_s, const void* keys, bool deep, const bh_nodes& nd, int order,
                     float theta, int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                     const uint32_t* sys = nullptr, const float4* sys_box = nullptr);
+// The whole build of a small set in one launch (false: the launch failed); the
+// group order is not made (see bh_groups_ordered).
+inline bool bh_small_set(int n, bool deep) { return n <= (deep ? 4096 : 8192); }
+bool launch_small_build(const float4* pos, int n, int n_leaf, int G, int curve, bool deep, const bh_nodes& nd,
+                        int64_t node_cap, void* keys, uint32_t* vals, float4* pos_s, int32_t* g_first, int32_t* g_count,
+                        bh_dev_ctrl* ctrl, cudaStream_t s);
+// Whether the groups of n particles are listed by cost for the walks: not where
+// every group has a block at once (the list costs a launch, 3 us).
+inline bool bh_groups_ordered(int n, int G) { return n > 16384 && n > 200 * G; }
 // One CTA per system: root cube, keys, stable radix sort and gather of each
 // system's particles (systems contiguous, each <= kBatchMaxN particles).
 constexpr int kBatchMaxN = 65536;

@@ -551,7 +551,8 @@ void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* b
     bh_launch_after(bh_group_mark_kernel, grid, 256, 0, s, nd, G, flags, ctrl);
     bh_launch_after(bh_flag_count_kernel, nblk, kFlagThreads, 0, s, flags, n, blk);
     bh_launch_after(bh_flag_write_kernel, nblk, kFlagThreads, 0, s, flags, n, blk, g_first, g_count, ctrl);
-    bh_launch_after(bh_group_order_kernel, std::min(grid, (n + 255) / 256), 256, 0, s, g_count, g_order, ctrl);
+    if (bh_groups_ordered(n, G))
+        bh_launch_after(bh_group_order_kernel, std::min(grid, (n + 255) / 256), 256, 0, s, g_count, g_order, ctrl);
 }
 
 // ------------------------------------------------------------ moments

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
         int ab = 0;
         if (lane == 0) ab = (int)*(volatile unsigned int*)&ctrl->abort;
         if (__shfl_sync(BH_FULL_MASK, ab, 0)) break;
-        g = P.g_order[g];
+        if (P.g_order) g = P.g_order[g];
         const int gb = P.g_first[g], gc = P.g_count[g], ge = gb + gc;
         const int tn = (gc + 31) >> 5;  // target slots in use (1..T)
         Layout L;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(256, bh_ws_min_blocks<T>()) bh_walk_ws_kernel(
             int ab = 0;
             if (lane == 0) ab = (int)*(volatile unsigned int*)&ctrl->abort;
             if (__shfl_sync(BH_FULL_MASK, ab, 0)) break;
-            g = P.g_order[g];
+            if (P.g_order) g = P.g_order[g];
             const int gb = P.g_first[g], gc = P.g_count[g], ge = gb + gc;
             unsigned int lo0 = 0xffffffffu, lo1 = 0xffffffffu, lo2 = 0xffffffffu, hi0 = 0u, hi1 = 0u, hi2 = 0u;
             for (int o = lane; o < gc; o += 32) {
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, false>()) bh_walk_t
         int ab = 0;
         if (lane == 0) ab = (int)*(volatile unsigned int*)&ctrl->abort;
         if (__shfl_sync(BH_FULL_MASK, ab, 0)) break;
-        g = P.g_order[g];
+        if (P.g_order) g = P.g_order[g];
         const int gb = P.g_first[g], gc = P.g_count[g], ge = gb + gc;
         const int tn = (gc + 31) >> 5;
         Layout L;
@@ -1266,7 +1266,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
     P.perm = perm;
     P.g_first = g_first;
     P.g_count = g_count;
-    P.g_order = g_order;
+    P.g_order = bh_groups_ordered(n, G) ? g_order : nullptr;
     P.rec = nd.rec;
     P.com_m = nd.com_m;
     P.seff = nd.seff;

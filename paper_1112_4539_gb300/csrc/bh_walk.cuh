@@ -96,7 +96,7 @@ struct WalkParams {
     const uint32_t* perm;
     const int32_t* g_first;
     const int32_t* g_count;
-    const int32_t* g_order;  // the groups by falling cost
+    const int32_t* g_order;  // the groups by falling cost (nullptr: in their own order)
     const int4* rec;
     const float4* com_m;
     const float* seff;

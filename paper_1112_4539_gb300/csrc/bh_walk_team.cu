@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(NW * 32, (T <= 3 ? 16 : 8) / NW) bh_walk_team_
         }
         __syncthreads();
         if (S.group < 0) break;
-        const int g = P.g_order[S.group];
+        const int g = P.g_order ? P.g_order[S.group] : S.group;
         const int gb = P.g_first[g], gc = P.g_count[g], ge = gb + gc;
         Layout L;
         {

@@ -384,7 +384,7 @@ int tree_force(bh_ctx* x, float eps, float* d_acc_pot, void* stream)
     if (!d_acc_pot || !aligned16(d_acc_pot) || !is_device_ptr(d_acc_pot, x->device)) return BH_ERR_INVALID;
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
-    bh::WalkLearned wl{x->mfeat, x->mlp, x->theta};
+    bh::WalkLearned wl{x->mfeat, x->mlp, x->theta, x->deep};
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
                              x->cfg.blocks_per_sm, (int)x->n, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);

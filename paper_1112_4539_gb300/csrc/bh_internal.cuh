@@ -427,6 +427,7 @@ struct WalkLearned {
     const float4* mfeat;
     const bh_mlp_dev* mlp;
     float theta_guard;
+    bool deep;  // 63-bit keys (more levels)
 };
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,

@@ -25,8 +25,9 @@
 // a pop the stack holds only levels below those popped, and the pushes of one
 // pop (<= 32 ranges) are the only entries of their levels.  Hence at most 33
 // ranges per level 1..21 are ever stored (21 = the deepest level of 63-bit
-// keys): kStackCap = 704 cannot overflow (overflow is still checked and
-// reported as BH_ERR_CAPACITY).
+// keys): kStackCap = 704 cannot overflow, nor kStackCapFlat = 336 on the 10
+// levels of 30-bit keys (overflow is still checked and reported as
+// BH_ERR_CAPACITY).
 #include "bh_walk.cuh"
 
 namespace bh {
@@ -35,14 +36,18 @@ namespace bh {
 #ifndef BH_WALK_MINB3
 #define BH_WALK_MINB3 4
 #endif
-template <int T, bool LEARNED>
+// Learned walk: with the stack of 30-bit keys four blocks fit the shared memory
+// (60.5 KB per block with the deep one), and 128 registers hold it without
+// spills: clumpy 2^22 12.72 -> 12.26 ms against three blocks of 156 registers.
+template <int T, bool LEARNED, int CAP = kStackCap>
 constexpr int bh_walk_min_blocks()
 {
-    return LEARNED ? (T <= 4 ? 3 : 2) : (T <= 1 ? 6 : T <= 2 ? 4 : T <= 3 ? BH_WALK_MINB3 : T <= 4 ? 3 : 2);
+    return LEARNED ? (T <= 3 && CAP < kStackCap ? 4 : T <= 4 ? 3 : 2) : (T <= 1 ? 6 : T <= 2 ? 4 : T <= 3 ? BH_WALK_MINB3 : T <= 4 ? 3 : 2);
 }
 
-template <int T, int ORDER, bool LEARNED>
-__global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
+// CAP: entries of a warp's stack
+template <int T, int ORDER, bool LEARNED, int CAP>
+__global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED, CAP>())
     bh_walk_kernel(WalkParams P)
 {
     bh_let_next_start();
@@ -50,11 +55,12 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    WarpSmem& S = reinterpret_cast<WarpSmem*>(smem_raw)[wib];
+    typedef WarpSmemOf<CAP> Smem;
+    Smem& S = reinterpret_cast<Smem*>(smem_raw)[wib];
     WarpQuad* Q = nullptr;
-    if (ORDER >= 2) Q = reinterpret_cast<WarpQuad*>(smem_raw + (size_t)nwarps * sizeof(WarpSmem)) + wib;
+    if (ORDER >= 2) Q = reinterpret_cast<WarpQuad*>(smem_raw + (size_t)nwarps * sizeof(Smem)) + wib;
     // learned criterion: the network (per block) and a feature staging area (per warp)
-    unsigned char* lbase = smem_raw + (size_t)nwarps * (sizeof(WarpSmem) + (ORDER >= 2 ? sizeof(WarpQuad) : 0));
+    unsigned char* lbase = smem_raw + (size_t)nwarps * (sizeof(Smem) + (ORDER >= 2 ? sizeof(WarpQuad) : 0));
     bh_mlp_dev* MW = reinterpret_cast<bh_mlp_dev*>(lbase);
     uint32_t* xs = reinterpret_cast<uint32_t*>(lbase + sizeof(bh_mlp_dev)) + wib * (32 * 8);
     // Kahan compensations (per warp, after the learned-criterion area)
@@ -202,7 +208,7 @@ __global__ void __launch_bounds__(128, bh_walk_min_blocks<T, LEARNED>())
             // ---- open: push child ranges
             const unsigned int om = __ballot_sync(BH_FULL_MASK, opn);
             const int npush = __popc(om);
-            if (sp + npush > kStackCap) {
+            if (sp + npush > CAP) {
                 overflow = true;
                 break;
             }
@@ -1209,15 +1215,15 @@ __global__ void bh_walk_reset_kernel(bh_dev_ctrl* c)
     c->n_pc = 0ull;
 }
 
-template <int T, int ORDER, bool LEARNED>
+template <int T, int ORDER, bool LEARNED, int CAP>
 static int bh_walk_launch_t(const WalkParams& P, int sm_count, int block_threads, int blocks_per_sm,
                             cudaStream_t s)
 {
     const int nw = block_threads / 32;
-    size_t smem = (size_t)nw * (sizeof(WarpSmem) + (ORDER >= 2 ? sizeof(WarpQuad) : 0));
+    size_t smem = (size_t)nw * (sizeof(WarpSmemOf<CAP>) + (ORDER >= 2 ? sizeof(WarpQuad) : 0));
     if (LEARNED) smem += sizeof(bh_mlp_dev) + (size_t)nw * 32 * 8 * sizeof(uint32_t);
     smem += (size_t)nw * bh_kahan_smem_bytes<T>();
-    auto kern = bh_walk_kernel<T, ORDER, LEARNED>;
+    auto kern = bh_walk_kernel<T, ORDER, LEARNED, CAP>;
     if (smem > 48 * 1024) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return BH_ERR_CUDA;
@@ -1231,7 +1237,7 @@ static int bh_walk_launch_t(const WalkParams& P, int sm_count, int block_threads
     return BH_OK;
 }
 
-template <bool LEARNED>
+template <bool LEARNED, int CAP = kStackCap>
 static int bh_walk_dispatch(const WalkParams& P, int order, int G, int sm_count, int block_threads,
                             int blocks_per_sm, cudaStream_t s)
 {
@@ -1239,19 +1245,19 @@ static int bh_walk_dispatch(const WalkParams& P, int order, int G, int sm_count,
     const int T = G <= 32 ? 1 : G <= 64 ? 2 : G <= 96 ? 3 : G <= 128 ? 4 : 8;
     if (order >= 2) {
         switch (T) {
-            case 1: return bh_walk_launch_t<1, 2, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-            case 2: return bh_walk_launch_t<2, 2, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-            case 3: return bh_walk_launch_t<3, 2, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-            case 4: return bh_walk_launch_t<4, 2, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-            default: return bh_walk_launch_t<8, 2, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
+            case 1: return bh_walk_launch_t<1, 2, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+            case 2: return bh_walk_launch_t<2, 2, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+            case 3: return bh_walk_launch_t<3, 2, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+            case 4: return bh_walk_launch_t<4, 2, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+            default: return bh_walk_launch_t<8, 2, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
         }
     }
     switch (T) {
-        case 1: return bh_walk_launch_t<1, 1, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-        case 2: return bh_walk_launch_t<2, 1, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-        case 3: return bh_walk_launch_t<3, 1, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-        case 4: return bh_walk_launch_t<4, 1, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
-        default: return bh_walk_launch_t<8, 1, LEARNED>(P, sm_count, block_threads, blocks_per_sm, s);
+        case 1: return bh_walk_launch_t<1, 1, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+        case 2: return bh_walk_launch_t<2, 1, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+        case 3: return bh_walk_launch_t<3, 1, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+        case 4: return bh_walk_launch_t<4, 1, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
+        default: return bh_walk_launch_t<8, 1, LEARNED, CAP>(P, sm_count, block_threads, blocks_per_sm, s);
     }
 }
 
@@ -1283,6 +1289,8 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
         P.mfeat = learned->mfeat;
         P.mlp = learned->mlp;
         P.theta_guard = learned->theta_guard;
+        if (!learned->deep)
+            return bh_walk_dispatch<true, kStackCapFlat>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
         return bh_walk_dispatch<true>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
     }
     if (walk_variant == BH_WALK_TMA && nd.wrec)

@@ -8,7 +8,8 @@
 
 namespace bh {
 
-constexpr int kStackCap = 704;
+constexpr int kStackCap = 704;      // see the stack bound in bh_walk.cu (21 levels)
+constexpr int kStackCapFlat = 336;  // the same bound for 10 levels (30-bit keys)
 constexpr int kTile = 64;              // sources per tile (one Kahan-compensated addition per tile)
 constexpr int kTilePairs = kTile / 2;  // a tile as even/odd source pairs
 constexpr int kRing = 2 * kTile;       // sources per ring (two tiles), stored as even/odd pairs
@@ -43,15 +44,17 @@ __host__ __device__ constexpr int bh_quad_unroll() { return LEARNED ? kQuadUnrol
 // Sources are staged negated and as pairs (ring positions 2p, 2p+1 side by
 // side) so that the interaction arithmetic runs on packed f32x2 operations:
 // one instruction computes the same step for two sources.
-struct WarpSmem {
+template <int CAP>
+struct WarpSmemOf {
     float gbox[8];              // the group's box: xmin, ymin, zmin, radius, xmax, ymax, zmax, -
     unsigned long long tot[2];  // interactions so far: particle-particle, particle-cell
-    uint32_t stack[kStackCap];  // (first node << 3) | (count - 1)
+    uint32_t stack[CAP];        // (first node << 3) | (count - 1)
     uint32_t staging[32];
     int2 leafq[64];             // pending particle ranges (first, count)
     float4 ra[kRing / 2];       // point sources: (-x, -x', -y, -y')
     float4 rb[kRing / 2];       //                (-z, -z', -m, -m')
 };
+typedef WarpSmemOf<kStackCap> WarpSmem;
 struct WarpQuad {               // quadrupole cells, pairs as above; Q = 3 I - T 1 (traceless), T = tr I
     float4 a[kRing / 2];        // (-x, -x', -y, -y')      centre of mass
     float4 b[kRing / 2];        // (-z, -z', -M, -M')
@@ -68,7 +71,11 @@ __device__ __forceinline__ void bh_put_point(float4* ra, float4* rb, int r, floa
     a[0] = -v.x; a[2] = -v.y;
     b[0] = -v.z; b[2] = -v.w;
 }
-__device__ __forceinline__ void bh_put_point(WarpSmem& S, int r, float4 v) { bh_put_point(S.ra, S.rb, r, v); }
+template <int CAP>
+__device__ __forceinline__ void bh_put_point(WarpSmemOf<CAP>& S, int r, float4 v)
+{
+    bh_put_point(S.ra, S.rb, r, v);
+}
 // cell with centre/mass cm and stored moments qb = (Ixx, Iyy, Izz, Ixy),
 // qc = (Ixz, Iyz, 1.5 T, 0.5 T): staged as the traceless Q = 3 I - T 1 and
 // -T eps^2 (see bh_pq2)

@@ -384,10 +384,10 @@ int tree_force(bh_ctx* x, float eps, float* d_acc_pot, void* stream)
     if (!d_acc_pot || !aligned16(d_acc_pot) || !is_device_ptr(d_acc_pot, x->device)) return BH_ERR_INVALID;
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
-    bh::WalkLearned wl{x->mfeat, x->mlp, x->theta, x->deep};
+    bh::WalkLearned wl{x->mfeat, x->mlp, x->theta};
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
-                             x->cfg.blocks_per_sm, (int)x->n, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
+                             x->cfg.blocks_per_sm, (int)x->n, x->deep, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     x->launches += bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
@@ -760,7 +760,7 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
                        x->cfg.curve, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count,
-                             x->cfg.block_threads, x->cfg.blocks_per_sm, N, s,
+                             x->cfg.block_threads, x->cfg.blocks_per_sm, N, x->deep, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     // init, batch sort, 4 tree, 3 or 4 groups, moments per level, 2 walk

@@ -427,12 +427,11 @@ struct WalkLearned {
     const float4* mfeat;
     const bh_mlp_dev* mlp;
     float theta_guard;
-    bool deep;  // 63-bit keys (more levels)
 };
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl,
-                int sm_count, int block_threads, int blocks_per_sm, int n, cudaStream_t s,
+                int sm_count, int block_threads, int blocks_per_sm, int n, bool deep, cudaStream_t s,
                 const WalkLearned* learned = nullptr, int walk_variant = 0);
 // failure-path self-tests: one bounded wait that nothing satisfies
 void launch_selftest_ring(bh_dev_ctrl* c, cudaStream_t s);

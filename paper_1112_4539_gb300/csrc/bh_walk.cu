@@ -1264,7 +1264,7 @@ static int bh_walk_dispatch(const WalkParams& P, int order, int G, int sm_count,
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl, int sm_count,
-                int block_threads, int blocks_per_sm, int n, cudaStream_t s, const WalkLearned* learned, int walk_variant)
+                int block_threads, int blocks_per_sm, int n, bool deep, cudaStream_t s, const WalkLearned* learned, int walk_variant)
 {
     bh_launch_after(bh_walk_reset_kernel, 1, 1, 0, s, ctrl);
     WalkParams P;
@@ -1289,7 +1289,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
         P.mfeat = learned->mfeat;
         P.mlp = learned->mlp;
         P.theta_guard = learned->theta_guard;
-        if (!learned->deep)
+        if (!deep)
             return bh_walk_dispatch<true, kStackCapFlat>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
         return bh_walk_dispatch<true>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
     }
@@ -1315,6 +1315,11 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
         const int rc = launch_walk_team(P, order, G, n, sm_count, s);
         if (rc <= 0) return rc;
     }
+    // one slot per lane: shared memory bounds the blocks per SM, five instead of
+    // four with the stack of 30-bit keys (Plummer 2^20, quadrupole,
+    // G = 32: 4.10 -> 3.95 ms)
+    if (G <= 32 && order >= 2 && !deep)
+        return bh_walk_launch_t<1, 2, false, kStackCapFlat>(P, sm_count, block_threads, blocks_per_sm, s);
     return bh_walk_dispatch<false>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
 }
 

@@ -35,7 +35,7 @@ def test_tiny_sets(n):
     _both(workloads.plummer(n, seed=3), 0.5, 0.0, order=2, group_size=96, leaf_size=16)
 
 
-@pytest.mark.parametrize("n,G", [(30011, 96), (60007, 96), (60007, 64), (90001, 32)])
+@pytest.mark.parametrize("n,G", [(30011, 96), (60007, 96), (60007, 64), (40001, 32)])
 @pytest.mark.parametrize("cfg", [dict(order=2, leaf_size=16), dict(order=1, leaf_size=64, curve=1),
                                  dict(order=2, leaf_size=8, max_level=21)])
 def test_both_block_sizes(n, G, cfg):

@@ -362,8 +362,8 @@ int tree_moments(bh_ctx* x, float theta, void* stream)
     cudaStream_t s = (cudaStream_t)stream;
     if (x->n > 0) {
         bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
-                           x->cfg.curve, x->ctrl, grid_for(x), s);
-        x->launches += bh::launches_moments(x->deep);
+                           x->cfg.curve, (int)x->n, x->ctrl, grid_for(x), s);
+        x->launches += bh::launches_moments((int)x->n, x->deep);
         if (x->mac_learned) {
             bh::launch_mac_nodefeat(x->nd, x->cfg.order, x->mfeat, x->ctrl, grid_for(x), s);
             x->launches += 1;
@@ -757,14 +757,15 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, (int32_t*)x->keys_alt,
                       x->ctrl, grid_for(x), s);
     bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
-                       x->cfg.curve, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
+                       x->cfg.curve, N, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count,
                              x->cfg.block_threads, x->cfg.blocks_per_sm, N, x->deep, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     // init, batch sort, 4 tree, 3 or 4 groups, moments per level, 2 walk
-    x->launches += 2 + 4 + (bh::bh_groups_ordered(N, x->cfg.group_size) ? 4 : 3) + bh::launches_moments(x->deep) + bh::kLaunchesForce;
+    x->launches += 2 + 4 + (bh::bh_groups_ordered(N, x->cfg.group_size) ? 4 : 3) +
+                   bh::launches_moments(N, x->deep) + bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
     x->theta = theta;

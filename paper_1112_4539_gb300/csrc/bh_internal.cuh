@@ -402,8 +402,11 @@ void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, u
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
                    int32_t* g_count, int32_t* g_order, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);
 void launch_moments(const float4* pos_s, const void* keys, bool deep, const bh_nodes& nd, int order,
-                    float theta, int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
+                    float theta, int fp64_threshold, int curve, int n, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                     const uint32_t* sys = nullptr, const float4* sys_box = nullptr);
+// Whether all levels' moments take one launch, and the launches of a set's moments.
+inline bool bh_moments_small(int n) { return n <= 8192; }
+inline int launches_moments(int n, bool deep) { return bh_moments_small(n) ? 1 : (deep ? 22 : 11) + 1; }  // large leaves, levels
 // The whole build of a small set in one launch (false: the launch failed); the
 // group order is not made (see bh_groups_ordered).
 inline bool bh_small_set(int n, bool deep) { return n <= (deep ? 4096 : 8192); }
@@ -462,7 +465,6 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
 
 // launches per call (deep = 63-bit keys: 8 sort passes, 22 levels)
 inline int launches_build(bool deep) { return deep ? 19 : 15; }  // init, bbox, keys, sort passes, 4 tree, 4 groups
-inline int launches_moments(bool deep) { return (deep ? 22 : 11) + 1; }  // large leaves, one per level
 constexpr int kLaunchesForce = 2;    // counter reset, walk
 constexpr int kLaunchesPWalk = 4;    // parent links, next links, counter reset, walk
 inline int launches_sph(bool deep) { return (deep ? 22 : 11) + 3; }  // node boxes per level, reset, two walks

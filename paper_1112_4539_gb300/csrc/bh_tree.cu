@@ -632,14 +632,10 @@ __device__ __forceinline__ float bh_warp_sumf(float x)
 // as it reads a child's.  Summed by one thread, a leaf of hundreds of
 // particles was the tail of the deepest level's launch.
 template <int ORDER>
-__global__ void __launch_bounds__(256) bh_bigleaf_moments_kernel(const float4* __restrict__ pos_s, bh_nodes nd,
-                                                                  const bh_dev_ctrl* __restrict__ c)
+__device__ __forceinline__ void bh_bigleaf_moments(const float4* __restrict__ pos_s, const bh_nodes& nd, int nn, int warp,
+                                                   int nw)
 {
-    bh_let_next_start();
-    bh_after_previous(pos_s, c);
     const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    const int nn = (int)c->n_nodes;
     // lane l of warp w examines nodes w + nw (l + 32 i): consecutive nodes go to
     // different warps, so the large leaves of a dense knot (adjacent in the
     // node order) spread over the grid instead of queueing in one warp
@@ -705,6 +701,16 @@ __global__ void __launch_bounds__(256) bh_bigleaf_moments_kernel(const float4* _
             }
         }
     }
+}
+
+template <int ORDER>
+__global__ void __launch_bounds__(256) bh_bigleaf_moments_kernel(const float4* __restrict__ pos_s, bh_nodes nd,
+                                                                  const bh_dev_ctrl* __restrict__ c)
+{
+    bh_let_next_start();
+    bh_after_previous(pos_s, c);
+    bh_bigleaf_moments<ORDER>(pos_s, nd, (int)c->n_nodes, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                              (gridDim.x * blockDim.x) >> 5);
 }
 
 template <typename R>
@@ -989,43 +995,74 @@ bh_moments_level_kernel(const float4* __restrict__ pos_s, const K* __restrict__ 
         bh_moment_node<ORDER, K, W>(pos_s, keys, nd, v, lev, theta, fp64_threshold, curve, gbox, sys, sys_box);
 }
 
-template <typename K>
-static void bh_moments_t(const float4* pos_s, const K* keys, const bh_nodes& nd, int order, float theta,
-                         int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
-                         const uint32_t* sys, const float4* sys_box)
+// All levels of a small set in one launch (the large leaves first) by one cluster
+// of eight blocks, with a cluster barrier between levels: their launches cost
+// more than their work.  Moments on GB300, a launch per level -> this: Plummer
+// 1000 monopole 30 -> 20 us, 4096 36 -> 28, clumpy 4096 quadrupole 39 -> 35, 8192
+// 41 -> 38, 16384 45 -> 46; 63-bit keys, 4096, 64 -> 39.  The four levels near the
+// root of any set in one such launch: 100003 71 -> 73 us, 2^24 437 -> 448, not kept.
+__device__ __forceinline__ void bh_cluster_sync()
 {
-    if (order >= 2) bh_launch_after(bh_bigleaf_moments_kernel<2>, grid, 256, 0, s, pos_s, nd, ctrl);
-    else bh_launch_after(bh_bigleaf_moments_kernel<1>, grid, 256, 0, s, pos_s, nd, ctrl);
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+template <int ORDER, typename K>
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512)
+bh_moments_cluster_kernel(const float4* __restrict__ pos_s, const K* __restrict__ keys, bh_nodes nd, float theta,
+                          int fp64_threshold, int curve, const bh_dev_ctrl* __restrict__ c,
+                          const uint32_t* __restrict__ sys, const float4* __restrict__ sys_box)
+{
+    bh_let_next_start();
+    bh_after_previous(pos_s, keys, c, sys, sys_box);
+    if (c->n_nodes == 0u) return;  // (every block alike)
+    const float4 gbox = make_float4(c->box[0], c->box[1], c->box[2], c->box[3]);
+    const int thread = blockIdx.x * 512 + threadIdx.x, threads = 8 * 512;
+    bh_bigleaf_moments<ORDER>(pos_s, nd, (int)c->n_nodes, thread >> 5, threads >> 5);
+    bh_cluster_sync();
     for (int lev = bh_key_traits<K>::kMaxLevel; lev >= 0; lev--) {
-        const bool warp = lev <= kWarpMomentLevels;
-        if (order >= 2) {
-            if (warp)
-                bh_launch_after(bh_moments_level_kernel<2, K, 32>, grid, 256, 0, s, pos_s, keys, nd, lev, theta, fp64_threshold,
-                                                                       curve, ctrl, sys, sys_box);
-            else
-                bh_launch_after(bh_moments_level_kernel<2, K, 1>, grid, 256, 0, s, 
-                    pos_s, keys, nd, lev, theta, fp64_threshold, curve, ctrl, sys, sys_box);
+        const int v0 = (int)c->level_offset[lev], v1 = (int)c->level_offset[lev + 1];
+        if (v0 == v1) continue;  // (every thread alike)
+        if (lev <= kWarpMomentLevels) {
+            for (int v = v0 + (thread >> 5); v < v1; v += threads >> 5)
+                bh_moment_node<ORDER, K, 32>(pos_s, keys, nd, v, lev, theta, fp64_threshold, curve, gbox, sys, sys_box);
         } else {
-            if (warp)
-                bh_launch_after(bh_moments_level_kernel<1, K, 32>, grid, 256, 0, s, pos_s, keys, nd, lev, theta, fp64_threshold,
-                                                                       curve, ctrl, sys, sys_box);
-            else
-                bh_launch_after(bh_moments_level_kernel<1, K, 1>, grid, 256, 0, s, 
-                    pos_s, keys, nd, lev, theta, fp64_threshold, curve, ctrl, sys, sys_box);
+            for (int v = v0 + thread; v < v1; v += threads)
+                bh_moment_node<ORDER, K, 1>(pos_s, keys, nd, v, lev, theta, fp64_threshold, curve, gbox, sys, sys_box);
         }
+        if (lev > 0) bh_cluster_sync();
+    }
+}
+
+template <int ORDER, typename K>
+static void bh_moments_t(const float4* pos_s, const K* keys, const bh_nodes& nd, float theta, int fp64_threshold,
+                         int curve, int n, bh_dev_ctrl* ctrl, int grid, cudaStream_t s, const uint32_t* sys,
+                         const float4* sys_box)
+{
+    if (bh_moments_small(n)) {
+        bh_launch_after(bh_moments_cluster_kernel<ORDER, K>, 8, 512, 0, s, pos_s, keys, nd, theta, fp64_threshold, curve,
+                        ctrl, sys, sys_box);
+        return;
+    }
+    bh_launch_after(bh_bigleaf_moments_kernel<ORDER>, grid, 256, 0, s, pos_s, nd, ctrl);
+    for (int lev = bh_key_traits<K>::kMaxLevel; lev >= 0; lev--) {
+        if (lev <= kWarpMomentLevels)
+            bh_launch_after(bh_moments_level_kernel<ORDER, K, 32>, grid, 256, 0, s, pos_s, keys, nd, lev, theta,
+                            fp64_threshold, curve, ctrl, sys, sys_box);
+        else
+            bh_launch_after(bh_moments_level_kernel<ORDER, K, 1>, grid, 256, 0, s, pos_s, keys, nd, lev, theta,
+                            fp64_threshold, curve, ctrl, sys, sys_box);
     }
 }
 
 void launch_moments(const float4* pos_s, const void* keys, bool deep, const bh_nodes& nd, int order, float theta,
-                    int fp64_threshold, int curve, bh_dev_ctrl* ctrl, int grid, cudaStream_t s, const uint32_t* sys,
-                    const float4* sys_box)
+                    int fp64_threshold, int curve, int n, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
+                    const uint32_t* sys, const float4* sys_box)
 {
-    if (deep)
-        bh_moments_t<bh_key64>(pos_s, (const bh_key64*)keys, nd, order, theta, fp64_threshold, curve, ctrl, grid, s,
-                               sys, sys_box);
-    else
-        bh_moments_t<uint32_t>(pos_s, (const uint32_t*)keys, nd, order, theta, fp64_threshold, curve, ctrl, grid, s,
-                               sys, sys_box);
+    auto run = [&](auto* k) {
+        if (order >= 2) bh_moments_t<2>(pos_s, k, nd, theta, fp64_threshold, curve, n, ctrl, grid, s, sys, sys_box);
+        else bh_moments_t<1>(pos_s, k, nd, theta, fp64_threshold, curve, n, ctrl, grid, s, sys, sys_box);
+    };
+    if (deep) run((const bh_key64*)keys);
+    else run((const uint32_t*)keys);
 }
 
 }  // namespace bh

@@ -156,16 +156,17 @@ int tree_moments(bh_ctx* ctx, float theta, void* stream);
  * tree_build); device status BH_ERR_CAPACITY or BH_ERR_DEVICE_TIMEOUT. */
 int tree_force(bh_ctx* ctx, float eps, float* d_acc_pot, void* stream);
 
-/* The paper's own walk (Sec. 4.4, Fig. 5, Appendix A): one thread per
- * particle follows the depth-first "more" (first child) and "next" (node
- * after the subtree) links from the root, with no stack.  For particle i a
+/* The paper's own walk (Sec. 4.4, Fig. 5, Appendix A): every particle
+ * reaches the nodes that the depth-first "more" (first child) and "next" (node
+ * after the subtree) links lead it to from the root, with its own decisions (a
+ * warp walks for 32 particles at a time).  For particle i a
  * node holding a single particle is a particle-particle term (skipped if it
  * is i); otherwise the node is accepted when |x_i - COM|^2 > S_eff (Eq. 2) and
  * it does not hold i, giving a particle-cell term (quadrupole when the
  * context's order is 2); a rejected leaf gives particle-particle terms with
  * its other members; a rejected internal node is entered.  The links are
- * derived from the current tree on each call.  FP32 terms, Kahan-compensated
- * runs of 32.  bh_stats then counts this walk's interactions.
+ * derived from the current tree on each call (for export).  FP32 terms,
+ * Kahan-compensated tiles of 32.  bh_stats then counts this walk's interactions.
  * eps >= 0: softening of Eq. (1).  flags: BH_PWALK_UNSOFTENED_CELLS applies
  * particle-cell terms with eps = 0, as the Appendix A kernel does;
  * BH_PWALK_INDIVIDUAL_SOFTENING uses the per-particle softening lengths set by
@@ -205,7 +206,8 @@ int tree_softening(bh_ctx* ctx, const float* d_eps, void* stream);
  * the cubic spline of Monaghan & Lattanzio (1985) of support h (unit
  * integral), FP32.  One warp walks the tree per particle group; a node is
  * skipped when its particles' bounding box is farther than the group's
- * largest radius from the group's box, so no neighbour is ever missed.
+ * largest radius from the group's box, so no neighbour is ever missed; groups
+ * with much work are walked again by a block of warps.
  * d_h: n radii in the caller's order, or NULL to use h for every particle.
  * d_count: n int32 neighbour counts (caller order, self excluded), or NULL.
  * d_rho: n float densities (caller order), or NULL.

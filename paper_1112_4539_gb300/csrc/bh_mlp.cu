@@ -230,8 +230,7 @@ constexpr int kOffB1 = BH_MLP_NH * BH_MLP_NF, kOffW2 = kOffB1 + BH_MLP_NH, kOffB
               kOffW3 = kOffB2 + BH_MLP_NH, kOffB3 = kOffW3 + BH_MLP_NH;
 constexpr int kAct = BH_MLP_NF + 4 * BH_MLP_NH + 1;  // floats of training scratch per sample (caller's buffer)
 constexpr int kRow = BH_MLP_NPARAM + 1;              // a block's partial sums: gradient, loss
-constexpr int kTrainSamples = 64;                    // samples per block and round
-constexpr int kTrainBlocks = 304;                    // most blocks (rows of partial sums)
+constexpr int kTrainBlocks = 304;                    // most blocks (rows of partial sums): two per SM
 
 // FP32 forward of one sample per thread (training path without gradients).
 __global__ void __launch_bounds__(256) bh_mlp_forward_kernel(const float* __restrict__ P, const float* __restrict__ X,
@@ -260,8 +259,8 @@ __global__ void __launch_bounds__(256) bh_mlp_forward_kernel(const float* __rest
     yhat[b] = y;
 }
 
-// Forward, backward and the weights' gradient of a mini-batch, 64 samples at
-// a time per block with every activation in shared memory.  Rounds of 64 are
+// Forward, backward and the weights' gradient of a mini-batch, kSamples (32 or
+// 64) at a time per block with every activation in shared memory.  Rounds are
 // dealt to the blocks in turn; a block keeps the gradient sums of its rounds
 // in registers and writes one row of kRow partial sums at the end.  rows == 1
 // (one block): the row is the gradient itself.
@@ -273,16 +272,18 @@ __global__ void __launch_bounds__(256) bh_mlp_forward_kernel(const float* __rest
 // 127 us (forward and backward 40 us, gradient 82 us, update 4 us), then 20.6 us
 // with this kernel and the sum of its rows, and 13.5 us with each of them
 // launched while its predecessor runs (bh_launch_after).
+template <int kSamples>
 struct TrainSmem {
     float p[BH_MLP_NPARAM + 3];                      // the parameters
     float w2t[BH_MLP_NH][BH_MLP_NH];                 // W2 transposed: [input][unit]
     float w2[BH_MLP_NH][BH_MLP_NH];                  // W2: [unit][input]
-    float x[kTrainSamples][BH_MLP_NF + 1];
-    float h1[kTrainSamples][BH_MLP_NH + 1], h2[kTrainSamples][BH_MLP_NH + 1];
-    float d1[kTrainSamples][BH_MLP_NH + 1], d2[kTrainSamples][BH_MLP_NH + 1];
-    float dy[kTrainSamples], l[kTrainSamples];
+    float x[kSamples][BH_MLP_NF + 1];
+    float h1[kSamples][BH_MLP_NH + 1], h2[kSamples][BH_MLP_NH + 1];
+    float d1[kSamples][BH_MLP_NH + 1], d2[kSamples][BH_MLP_NH + 1];
+    float dy[kSamples], l[kSamples];
 };
 
+template <int kSamples>
 __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __restrict__ P,
                                                                 const float* __restrict__ X,
                                                                 const float* __restrict__ Y,
@@ -291,7 +292,8 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
                                                                 float* __restrict__ loss)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    TrainSmem<kSamples>& S = *reinterpret_cast<TrainSmem<kSamples>*>(smem_raw);
+    constexpr int kUnits = kSamples / 8;  // hidden units per thread
     const int tid = threadIdx.x;
     bh_let_next_start();
     // the first round's samples, which no kernel of this call writes, are
@@ -304,7 +306,7 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
 #pragma unroll
         for (int k = 0; k < BH_MLP_NF; k++) x0[k] = in ? X[at * BH_MLP_NF + k] : 0.f;
     };
-    if (tid < kTrainSamples) fetch(blockIdx.x * kTrainSamples + tid);
+    if (tid < kSamples) fetch(blockIdx.x * kSamples + tid);
     bh_after_previous(P, rows, loss);
     for (int i = tid; i < BH_MLP_NPARAM; i += 256) S.p[i] = P[i];
     for (int i = tid; i < BH_MLP_NH * BH_MLP_NH; i += 256) {
@@ -312,7 +314,7 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
         S.w2[i / BH_MLP_NH][i % BH_MLP_NH] = w;
         S.w2t[i % BH_MLP_NH][i / BH_MLP_NH] = w;
     }
-    const int s = tid & 63, u0 = (tid >> 6) * 8;  // sample, first of 8 units (a warp shares u0)
+    const int s = tid % kSamples, u0 = tid / kSamples * kUnits;  // sample, first unit (a warp shares u0)
     // weight gradient of layer 2: units ja + 8 a, inputs ka + 8 b, samples q, q + 4, ...
     const int ja = (tid & 63) >> 3, ka = tid & 7, q = tid >> 6;
     float g2[4][4];
@@ -321,12 +323,12 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
 #pragma unroll
         for (int b = 0; b < 4; b++) g2[a][b] = 0.f;
     float ge[2] = {0.f, 0.f};  // the thread's one or two other outputs
-    const int nround = (B + kTrainSamples - 1) / kTrainSamples;
+    const int nround = (B + kSamples - 1) / kSamples;
     for (int round = blockIdx.x; round < nround; round += gridDim.x) {
-        const int b = round * kTrainSamples + s;
+        const int b = round * kSamples + s;
         const bool in = b < B;
         __syncthreads();
-        if (tid < kTrainSamples) {
+        if (tid < kSamples) {
             if (round != blockIdx.x) fetch(b);
 #pragma unroll
             for (int k = 0; k < BH_MLP_NF; k++) S.x[s][k] = x0[k];
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
 #pragma unroll
             for (int k = 0; k < BH_MLP_NF; k++) x[k] = S.x[s][k];
 #pragma unroll
-            for (int j = u0; j < u0 + 8; j++) {
+            for (int j = u0; j < u0 + kUnits; j++) {
                 float a = S.p[kOffB1 + j];
 #pragma unroll
                 for (int k = 0; k < BH_MLP_NF; k++) a = fmaf(S.p[j * BH_MLP_NF + k], x[k], a);
@@ -348,23 +350,25 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
         __syncthreads();
         // layer 2
         {
-            float a[8];
+            float a[kUnits];
 #pragma unroll
-            for (int j = 0; j < 8; j++) a[j] = S.p[kOffB2 + u0 + j];
+            for (int j = 0; j < kUnits; j++) a[j] = S.p[kOffB2 + u0 + j];
 #pragma unroll 8
             for (int k = 0; k < BH_MLP_NH; k++) {
                 const float h = S.h1[s][k];
-                const float4 w0 = *reinterpret_cast<const float4*>(&S.w2t[k][u0]);
-                const float4 w1 = *reinterpret_cast<const float4*>(&S.w2t[k][u0 + 4]);
-                a[0] = fmaf(w0.x, h, a[0]); a[1] = fmaf(w0.y, h, a[1]); a[2] = fmaf(w0.z, h, a[2]); a[3] = fmaf(w0.w, h, a[3]);
-                a[4] = fmaf(w1.x, h, a[4]); a[5] = fmaf(w1.y, h, a[5]); a[6] = fmaf(w1.z, h, a[6]); a[7] = fmaf(w1.w, h, a[7]);
+#pragma unroll
+                for (int j = 0; j < kUnits; j += 4) {
+                    const float4 w = *reinterpret_cast<const float4*>(&S.w2t[k][u0 + j]);
+                    a[j] = fmaf(w.x, h, a[j]); a[j + 1] = fmaf(w.y, h, a[j + 1]);
+                    a[j + 2] = fmaf(w.z, h, a[j + 2]); a[j + 3] = fmaf(w.w, h, a[j + 3]);
+                }
             }
 #pragma unroll
-            for (int j = 0; j < 8; j++) S.h2[s][u0 + j] = fmaxf(a[j], 0.f);
+            for (int j = 0; j < kUnits; j++) S.h2[s][u0 + j] = fmaxf(a[j], 0.f);
         }
         __syncthreads();
         // output, loss and its derivative
-        if (tid < kTrainSamples) {
+        if (tid < kSamples) {
             float y = S.p[kOffB3];
 #pragma unroll 8
             for (int k = 0; k < BH_MLP_NH; k++) y = fmaf(S.p[kOffW3 + k], S.h2[s][k], y);
@@ -377,27 +381,29 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
         {
             const float dy = S.dy[s];
 #pragma unroll
-            for (int j = u0; j < u0 + 8; j++) S.d2[s][j] = S.h2[s][j] > 0.f ? dy * S.p[kOffW3 + j] : 0.f;
+            for (int j = u0; j < u0 + kUnits; j++) S.d2[s][j] = S.h2[s][j] > 0.f ? dy * S.p[kOffW3 + j] : 0.f;
         }
         __syncthreads();
         {
-            float d[8];
+            float d[kUnits];
 #pragma unroll
-            for (int k = 0; k < 8; k++) d[k] = 0.f;
+            for (int k = 0; k < kUnits; k++) d[k] = 0.f;
 #pragma unroll 8
             for (int j = 0; j < BH_MLP_NH; j++) {
                 const float e = S.d2[s][j];
-                const float4 w0 = *reinterpret_cast<const float4*>(&S.w2[j][u0]);
-                const float4 w1 = *reinterpret_cast<const float4*>(&S.w2[j][u0 + 4]);
-                d[0] = fmaf(e, w0.x, d[0]); d[1] = fmaf(e, w0.y, d[1]); d[2] = fmaf(e, w0.z, d[2]); d[3] = fmaf(e, w0.w, d[3]);
-                d[4] = fmaf(e, w1.x, d[4]); d[5] = fmaf(e, w1.y, d[5]); d[6] = fmaf(e, w1.z, d[6]); d[7] = fmaf(e, w1.w, d[7]);
+#pragma unroll
+                for (int k = 0; k < kUnits; k += 4) {
+                    const float4 w = *reinterpret_cast<const float4*>(&S.w2[j][u0 + k]);
+                    d[k] = fmaf(e, w.x, d[k]); d[k + 1] = fmaf(e, w.y, d[k + 1]);
+                    d[k + 2] = fmaf(e, w.z, d[k + 2]); d[k + 3] = fmaf(e, w.w, d[k + 3]);
+                }
             }
 #pragma unroll
-            for (int k = 0; k < 8; k++) S.d1[s][u0 + k] = S.h1[s][u0 + k] > 0.f ? d[k] : 0.f;
+            for (int k = 0; k < kUnits; k++) S.d1[s][u0 + k] = S.h1[s][u0 + k] > 0.f ? d[k] : 0.f;
         }
         // gradient of W2 (d2 and h1 are complete)
 #pragma unroll 4
-        for (int i = q; i < kTrainSamples; i += 4) {
+        for (int i = q; i < kSamples; i += 4) {
             float d[4], h[4];
 #pragma unroll
             for (int a = 0; a < 4; a++) {
@@ -419,14 +425,14 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
             else { f = &S.d2[0][tid - 224]; g = nullptr; }
             float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll 8
-            for (int i = 0; i < kTrainSamples; i += 2) {
+            for (int i = 0; i < kSamples; i += 2) {
                 acc0 = fmaf(f[i * (BH_MLP_NH + 1)], g ? g[i * gs] : 1.0f, acc0);
                 acc1 = fmaf(f[(i + 1) * (BH_MLP_NH + 1)], g ? g[(i + 1) * gs] : 1.0f, acc1);
             }
             ge[0] += acc0 + acc1;
             if (tid < BH_MLP_NH + 2) {
                 acc0 = acc1 = 0.f;
-                for (int i = 0; i < kTrainSamples; i += 2) {
+                for (int i = 0; i < kSamples; i += 2) {
                     const float u = tid < BH_MLP_NH ? S.h2[i][tid] : 1.0f, w = tid < BH_MLP_NH ? S.h2[i + 1][tid] : 1.0f;
                     acc0 = fmaf(tid == BH_MLP_NH + 1 ? S.l[i] : S.dy[i], u, acc0);
                     acc1 = fmaf(tid == BH_MLP_NH + 1 ? S.l[i + 1] : S.dy[i + 1], w, acc1);
@@ -437,7 +443,8 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
     }
     // the four sample slices of W2's gradient, then the row
     __syncthreads();
-    float* red = &S.h1[0][0];  // [4][1024] over h1, h2 (4224 floats)
+    float* red = &S.h1[0][0];  // [4][1024] over h1, h2, d1, d2
+    static_assert(4 * kSamples * (BH_MLP_NH + 1) >= 4096, "room for the slices");
 #pragma unroll
     for (int a = 0; a < 4; a++)
 #pragma unroll
@@ -587,10 +594,31 @@ int mac_label(const float4* pos_s, const uint32_t* perm, const int32_t* g_first,
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
 
-static bool train_smem_ok()
+// A block's share of a mini-batch of B samples per round, and the blocks.
+struct TrainPlan {
+    void (*kernel)(const float*, const float*, const float*, const int32_t*, long long, int, long long, float, float*,
+                   float*);
+    int blocks;
+    size_t smem;
+};
+
+template <int kSamples>
+static TrainPlan train_plan(long long B)
 {
-    return cudaFuncSetAttribute(bh_mlp_batch_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(TrainSmem)) == cudaSuccess;
+    TrainPlan t{bh_mlp_batch_grad_kernel<kSamples>, (int)std::min<long long>((B + kSamples - 1) / kSamples, kTrainBlocks),
+                sizeof(TrainSmem<kSamples>)};
+    if (cudaFuncSetAttribute(t.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t.smem) != cudaSuccess)
+        t.blocks = 0;
+    return t;
+}
+
+// 32 samples per block halve each phase of a round, and give twice the rows to
+// sum.  They pay while every block has an SM to itself (152 x 32 = 4864
+// samples).  Microseconds per step with 32 | 64 on GB300: 512 samples 10.5 |
+// 13.0, 2048 11.6 | 13.6, 4096 10.8 | 14.4, 5000 16.0 | 14.4, 8192 16.4 | 13.5.
+static TrainPlan train_plan_for(long long B)
+{
+    return B <= kTrainBlocks / 2 * 32 ? train_plan<32>(B) : train_plan<64>(B);
 }
 
 int mlp_train(const float* X, const float* Y, const int32_t* order, long long n, float* P, float* adam_m,
@@ -600,19 +628,17 @@ int mlp_train(const float* X, const float* Y, const int32_t* order, long long n,
     if (batch < 1 || n < 1 || steps < 0) return BH_ERR_INVALID;
     const long long need = (long long)batch * kAct + BH_MLP_NPARAM;
     if (work_floats < need) return BH_ERR_TOO_LARGE;
-    const int blocks = std::min((batch + kTrainSamples - 1) / kTrainSamples, kTrainBlocks);
-    if (!train_smem_ok()) return BH_ERR_CUDA;
+    const TrainPlan plan = train_plan_for(batch);
+    if (plan.blocks == 0) return BH_ERR_CUDA;
     for (long long st = 0; st < steps; st++) {
         const long long i0 = ((t0 + st) * (long long)batch) % n;
         float* l = loss ? loss + st : nullptr;
         if (st == 0)  // its samples may still be in the making
-            bh_mlp_batch_grad_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, X, Y, order, i0, batch, n, under_w, work,
-                                                                            l);
+            plan.kernel<<<plan.blocks, 256, plan.smem, s>>>(P, X, Y, order, i0, batch, n, under_w, work, l);
         else
-            bh_launch_after(bh_mlp_batch_grad_kernel, blocks, 256, sizeof(TrainSmem), s, P, X, Y, order, i0, batch, n,
-                            under_w, work, l);
-        bh_launch_after(bh_mlp_update_kernel, (kRow + 31) / 32, 256, 0, s, work, blocks, nullptr, l, P, adam_m, adam_v,
-                        t0 + st + 1, lr, 0.9f, 0.999f, 1e-8f);
+            bh_launch_after(plan.kernel, plan.blocks, 256, plan.smem, s, P, X, Y, order, i0, batch, n, under_w, work, l);
+        bh_launch_after(bh_mlp_update_kernel, (kRow + 31) / 32, 256, 0, s, work, plan.blocks, nullptr, l, P, adam_m,
+                        adam_v, t0 + st + 1, lr, 0.9f, 0.999f, 1e-8f);
     }
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
@@ -623,14 +649,14 @@ int mlp_grad(const float* P, const float* X, const float* Y, long long n, float 
     const long long need = n * kAct;
     if (work_floats < need) return BH_ERR_TOO_LARGE;
     if (n > (1ll << 30)) return BH_ERR_TOO_LARGE;
-    // rows of partial sums fit in n * kAct floats whenever there are two or more (n > 64)
-    const int blocks = (int)std::min<long long>((n + kTrainSamples - 1) / kTrainSamples, kTrainBlocks);
-    if (!train_smem_ok()) return BH_ERR_CUDA;
-    bh_mlp_batch_grad_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, X, Y, nullptr, 0, (int)n, n, under_w,
-                                                                    blocks > 1 ? work : grad, loss);
-    if (blocks > 1)
-        bh_mlp_update_kernel<<<(kRow + 31) / 32, 256, 0, s>>>(work, blocks, grad, loss, nullptr, nullptr, nullptr, 1,
-                                                              0.f, 0.9f, 0.999f, 1e-8f);
+    // rows of partial sums fit in n * kAct floats whenever there are two or more (n > 32)
+    const TrainPlan plan = train_plan_for(n);
+    if (plan.blocks == 0) return BH_ERR_CUDA;
+    plan.kernel<<<plan.blocks, 256, plan.smem, s>>>(P, X, Y, nullptr, 0, (int)n, n, under_w,
+                                                    plan.blocks > 1 ? work : grad, loss);
+    if (plan.blocks > 1)
+        bh_mlp_update_kernel<<<(kRow + 31) / 32, 256, 0, s>>>(work, plan.blocks, grad, loss, nullptr, nullptr, nullptr,
+                                                              1, 0.f, 0.9f, 0.999f, 1e-8f);
     return cudaGetLastError() == cudaSuccess ? BH_OK : BH_ERR_CUDA;
 }
 

@@ -11,15 +11,16 @@
 // (Sec. 7, after Saitoh & Makino 2010).
 //
 // FP64 is bound by the FP64 pipe (2 lanes per clock and SM on GB300, 1/64 of
-// FP32), so what counts is the FP64 instructions per pair: 18 here (3 for the
-// difference, 3 for r^2 + eps^2, 5 for its inverse square root, 7 for the
+// FP32), so what counts is the FP64 instructions per pair: 15 here (3 for the
+// difference, 3 for r^2 + eps^2, 2 for its inverse square root, 7 for the
 // sums).  Sources are converted once per tile instead of once per pair, and
-// 1/sqrt is a hardware estimate with one step of Householder's third-order
-// iteration instead of a correctly rounded square root and division.  4096
-// targets x 2^20 sources: 244.6 ms with those, 139.5 ms now (19 flops per pair
-// counted: 0.58 TFLOP/s), the same error against FP64 sums by PyTorch
-// (2.5e-16).  FP32, 16384 targets x 2^18 sources: one source at a time with the
-// self test on every pair 2.94 ms, packed pairs 1.77 ms (46 TFLOP/s).
+// 1/sqrt does all but its last two steps on the other pipes (bh_rsqrt64).
+// 4096 targets x 2^20 sources: 244.6 ms with a correctly rounded square root
+// and division, 139.5 ms with an FP64 iteration (18 instructions per pair),
+// 113.7 ms now (19 flops per pair counted: 0.72 TFLOP/s), the same error
+// against FP64 sums by PyTorch (2.5e-16).  FP32, 16384 targets x 2^18 sources:
+// one source at a time with the self test on every pair 2.94 ms, packed pairs
+// 1.77 ms (46 TFLOP/s).
 #include <type_traits>
 
 #include "bh_walk.cuh"
@@ -37,17 +38,49 @@ __device__ __forceinline__ void bh_kahan_r(R& s, R& c, R v)
     s = t;
 }
 
-// x^-1/2: the hardware's estimate y (about 20 bits) and one step of the
-// third-order iteration y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2, whose error is
-// 5 e^3 / 16, below 2^-56.  Zero and infinity keep their estimates (inf, 0).
+// x^-1/2 with two FP64 instructions, everything else on the FP32 and integer
+// pipes (64 of their instructions take the time of one of FP64).  With
+// x = 4^k f, 1 <= f < 4, and y0 the FP32 estimate of f^-1/2, whose square y0^2
+// has 48 bits and so is exact as a double,
+//   f^-1/2 = y0 (1 + e/2 + 3 e^2/8 + ...),  e = 1 - f y0^2, |e| < 2^-21,
+// and the next term is below 2^-64.  The quadratic term comes from an FP32 e
+// (error 2^-45, f and y0^2 split in two floats each) and enters the constant of
+// the FP64 one, d = (1 - 2^-28 + 3 e^2/4) - f y0^2, one fma.  The offset 2^-28
+// keeps that constant below 1, where doubles lie 2^-53 apart, and goes back
+// exactly: y0 (1 + 2^-29) has 53 bits, so that x^-1/2 = y0 (1 + 2^-29) + y0 d/2
+// is the other fma.  Error at most 1.25 2^-53, rms 0.46 2^-53 (4 million x over
+// all exponents on the host, any y0 within its bound; an FP64 third-order step
+// from a 20-bit estimate, 5 FP64 instructions, has 1.50 and 0.48).
+// Zero and denormal x give inf, inf gives 0.
 __device__ __forceinline__ double bh_rsqrt64(double x)
 {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t fe = 0x40000000u - ((hi & 0x100000u) << 3);      // f = fh + fl: exponent bits of fh
+    const float fh = __uint_as_float(((hi << 3 | lo >> 29) & 0x7fffffu) | fe);
+    const uint32_t ge = fe - (23u << 23);                           // the next 23 bits lie 23 places lower
+    const float fl = __fsub_rn(__uint_as_float(((lo << 3) >> 9) | ge), __uint_as_float(ge));
+    float y0;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(fh));
+    const uint32_t yb = __float_as_uint(y0), ye = yb >> 23, ym = (yb & 0x7fffffu) | 0x800000u;
+    // e in FP32, and 3 e^2 / 4 in units of 2^-53
+    const float ph = __fmul_rn(y0, y0), pl = __fmaf_rn(y0, y0, -ph);
+    const float e = __fmaf_rn(-fl, ph, __fmaf_rn(-fh, pl, __fmaf_rn(-fh, ph, 1.0f)));
+    const uint32_t q = __float_as_uint(__fmaf_rn(__fmul_rn(e, e), 0.75f * 9007199254740992.0f, 8388608.0f)) - 0x4b000000u;
+    const double c = __hiloint2double(0x3fefffff, (int)(0xfe000000u + q));
+    // y0^2: the mantissa's square with its leading bit at bit 52, where it counts into the exponent
+    unsigned long long sq = (unsigned long long)ym * ym;
+    const uint32_t top = (uint32_t)(sq >> 47);
+    sq <<= 6 - top;
+    const double yy = __hiloint2double((int)((uint32_t)(sq >> 32) + ((2 * ye + 768 + top) << 20)), (int)(uint32_t)sq);
+    const double f = __hiloint2double((int)((hi & 0xfffffu) | (0x40000000u - (hi & 0x100000u))), (int)lo);
+    const double d = __fma_rn(-f, yy, c);
+    const uint32_t h = (yb >> 3) + (1408u << 20) - (((hi + 0x100000u) >> 21) << 20);  // 2^-k y0
+    const double r = __fma_rn(__hiloint2double((int)(h - 0x100000u), (int)(yb << 29)), d,
+                              __hiloint2double((int)h, (int)((yb << 29) + ym)));
+    if (hi - 0x100000u < 0x7fe00000u) return r;  // a normal number
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
-    const double r = __fma_rn(y, __dmul_rn(e, __fma_rn(0.375, e, 0.5)), y);
-    const int h = __double2hiint(y);
-    return (h == 0 || h == 0x7ff00000) ? y : r;
+    return y;
 }
 
 template <bool ATOMIC, bool SYM>

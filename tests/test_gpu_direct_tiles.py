@@ -51,3 +51,23 @@ def test_tiles(n, precision, kind):
     got = out.cpu().numpy().astype(np.longdouble)
     assert (np.abs(got - want) <= TOL[precision] * mag + np.longdouble(1e-300)).all()
 
+
+
+@pytest.mark.parametrize("scale", [-120, -101, -37, 0, 23, 60])
+def test_inverse_root(scale):
+    """FP64, one source and one target per sum: every exponent and mantissa pattern of r^2, nothing to average over.
+    With u = 2^-53, r^2 is off by at most 5 u (differences 2 u, three fused adds), its inverse root by 2.5 u + 1.5 u,
+    the potential by 1 u more, the force by 3 x 4 u and 5 roundings."""
+    import paper_1112_4539_gb300 as bh
+    rng = np.random.Generator(np.random.Philox(key=scale + 500))
+    n = 500
+    src, tgt = np.zeros((1, 4), np.float32), np.zeros((n, 4), np.float32)
+    src[0, 3] = 1.0
+    tgt[:, :3] = np.ldexp(rng.uniform(-2, 2, (n, 3)), scale + rng.integers(-4, 5, (n, 1)))
+    tgt[:4, :3] = np.ldexp(np.array([[1, 0, 0], [0, 2, 0], [1, 1, 0], [np.nextafter(np.float32(2), 0), 0, 0]]), scale)
+    want, mag = _reference(src, tgt, np.full(n, -1), np.longdouble(0))
+    d = [torch.from_numpy(a).cuda() for a in (src, tgt)]
+    out = torch.empty((n, 4), device="cuda", dtype=torch.float64)
+    assert bh.direct_force(d[0], d[1], torch.full((n,), -1, dtype=torch.int64, device="cuda"), 0.0, out, 64) == 0
+    err = np.abs(out.cpu().numpy().astype(np.longdouble) - want) * 2.0 ** 53
+    assert (err[:, :3] <= 18 * mag[:, :3]).all() and (err[:, 3] <= 6 * mag[:, 3]).all()

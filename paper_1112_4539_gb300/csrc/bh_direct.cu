@@ -83,7 +83,10 @@ __device__ __forceinline__ double bh_rsqrt64(double x)
     return y;
 }
 
-template <bool ATOMIC, bool SYM>
+// NARROW: a block takes 32 targets, one per lane, and its warps share each tile
+// of sources, 32 each; their sums are put together at the end with their
+// compensations.
+template <bool NARROW, bool ATOMIC, bool SYM>
 __global__ void __launch_bounds__(kDirThreads)
 bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __restrict__ tgt,
                    const int64_t* __restrict__ self, int n_tgt, double eps2, bh_double4* __restrict__ out, int chunk,
@@ -91,7 +94,9 @@ bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __re
 {
     __shared__ bh_double4 tile[kDirThreads];
     __shared__ double tile_e[SYM ? kDirThreads : 1];  // eps_j^2 / 2
-    const int i = blockIdx.x * kDirThreads + threadIdx.x;
+    constexpr int kRun = NARROW ? 32 : kDirThreads;  // sources of a tile that a warp takes
+    const int lane = threadIdx.x & 31, first = NARROW ? threadIdx.x - lane : 0;
+    const int i = NARROW ? blockIdx.x * 32 + lane : blockIdx.x * kDirThreads + threadIdx.x;
     const bool valid = i < n_tgt;
     float4 pt = make_float4(0.f, 0.f, 0.f, 0.f);
     long long sf = -1;
@@ -118,10 +123,10 @@ bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __re
         }
         __syncthreads();
         double tx = 0, ty = 0, tz = 0, tp = 0;
-        const int skip = (sf >= base && sf < base + kDirThreads) ? (int)(sf - base) : -1;
+        const int skip = (sf >= base + first && sf < base + first + kRun) ? (int)(sf - base) : -1;
         auto pairs = [&](auto with_self) {
 #pragma unroll 4
-            for (int k = 0; k < kDirThreads; k++) {
+            for (int k = first; k < first + kRun; k++) {
                 const bh_double4 s = tile[k];
                 const double dx = s.x - xi, dy = s.y - yi, dz = s.z - zi;
                 double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, __fma_rn(dz, dz, SYM ? hi + tile_e[k] : eps2)));
@@ -146,6 +151,21 @@ bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __re
         bh_kahan_r<double>(az, cz, tz);
         bh_kahan_r<double>(ph, cp, tp);
         __syncthreads();
+    }
+    if (NARROW) {
+        __shared__ bh_double4 rest[NARROW ? kDirThreads : 1];
+        tile[threadIdx.x] = bh_double4{ax, ay, az, ph};
+        rest[threadIdx.x] = bh_double4{cx, cy, cz, cp};
+        __syncthreads();
+        if (first != 0 || !valid) return;
+        for (int k = lane + 32; k < kDirThreads; k += 32) {
+            const bh_double4 v = tile[k], c = rest[k];
+            cx += c.x; cy += c.y; cz += c.z; cp += c.w;
+            bh_kahan_r<double>(ax, cx, v.x);
+            bh_kahan_r<double>(ay, cy, v.y);
+            bh_kahan_r<double>(az, cz, v.z);
+            bh_kahan_r<double>(ph, cp, v.w);
+        }
     }
     if (!valid) return;
     const double rx = ax - cx, ry = ay - cy, rz = az - cz, rp = ph - cp;
@@ -255,14 +275,22 @@ int launch_direct(const float4* src, int n_src, const float4* tgt, const int64_t
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tblocks = (n_tgt + kDirThreads - 1) / kDirThreads;
     // split the sources when the targets alone give under ~8 blocks per SM
-    int split = 1;
-    if (tblocks < 8 * sms && n_src > 4 * kDirThreads) {
-        split = (8 * sms + tblocks - 1) / tblocks;
-        split = min(split, (n_src + 4 * kDirThreads - 1) / (4 * kDirThreads));
-        split = max(split, 1);
-    }
+    int tblocks = 0, split = 1;
+    auto plan = [&](int targets, int most) {
+        tblocks = (n_tgt + targets - 1) / targets;
+        split = tblocks < 8 * sms ? max(min((8 * sms + tblocks - 1) / tblocks, most), 1) : 1;
+    };
+    const int most = n_src / (4 * kDirThreads) + (n_src % (4 * kDirThreads) != 0);
+    plan(kDirThreads, most);
+    // FP64 with less than two such blocks per SM: 32 targets per block, in as
+    // many partial sums as above, or 16 (which the shorter plain sums make up
+    // for), of a tile of sources at least.  Microseconds with 256 targets per
+    // block | 32: 1000 targets x 4000 sources 1073 | 162.  Error against FP64
+    // sums by PyTorch: 1.3e-16 at 256 x 1024 (2.8e-16 before), 1.4e-16
+    // (1.6e-16) at 256 x 2^14, 3.3e-16 (4.6e-16) at 256 x 2^18.
+    const bool narrow = precision == 64 && (long long)tblocks * split < 2 * sms;
+    if (narrow) plan(32, max(most, min(16, n_src / kDirThreads + (n_src % kDirThreads != 0))));
     const int chunk = ((n_src + split - 1) / split + kDirThreads - 1) / kDirThreads * kDirThreads;
     split = max(1, (n_src + chunk - 1) / max(chunk, 1));
     const dim3 grid(tblocks, split);
@@ -279,8 +307,13 @@ int launch_direct(const float4* src, int n_src, const float4* tgt, const int64_t
     };
     const bool at = split > 1, normal = !sym && (float)(eps * eps) >= 1.17549435e-38f;
     if (precision == 64) {
-        if (sym) at ? launch64(bh_direct64_kernel<true, true>) : launch64(bh_direct64_kernel<false, true>);
-        else at ? launch64(bh_direct64_kernel<true, false>) : launch64(bh_direct64_kernel<false, false>);
+        auto choose = [&](auto form) {
+            constexpr bool N = decltype(form)::value;
+            if (sym) at ? launch64(bh_direct64_kernel<N, true, true>) : launch64(bh_direct64_kernel<N, false, true>);
+            else at ? launch64(bh_direct64_kernel<N, true, false>) : launch64(bh_direct64_kernel<N, false, false>);
+        };
+        if (narrow) choose(std::true_type());
+        else choose(std::false_type());
     } else if (sym) {
         at ? launch32(bh_direct32_kernel<true, true, false>) : launch32(bh_direct32_kernel<false, true, false>);
     } else if (normal) {

@@ -71,3 +71,24 @@ def test_inverse_root(scale):
     assert bh.direct_force(d[0], d[1], torch.full((n,), -1, dtype=torch.int64, device="cuda"), 0.0, out, 64) == 0
     err = np.abs(out.cpu().numpy().astype(np.longdouble) - want) * 2.0 ** 53
     assert (err[:, :3] <= 18 * mag[:, :3]).all() and (err[:, 3] <= 6 * mag[:, 3]).all()
+
+
+@pytest.mark.parametrize("n,nt", [(257, 77825), (1025, 38912), (1025, 38656), (9000, 33)])
+@pytest.mark.parametrize("kind", ["softened", "symmetrized"])
+def test_wide(n, nt, kind):
+    """FP64, 256 targets per block (from two blocks per SM on) and 32 with sources for several tiles each."""
+    import paper_1112_4539_gb300 as bh
+    pos = workloads.plummer(n, seed=n)
+    tgt = np.concatenate([pos, workloads.plummer(nt, seed=98)])[:nt]
+    idx = np.where(np.arange(nt) < n, np.arange(nt), -1)
+    at = np.unique(np.concatenate([np.arange(16), np.linspace(0, nt - 1, 200).astype(int)]))
+    es, et = workloads.softening_lengths(n, 0.01), workloads.softening_lengths(nt, 0.01, seed=5)
+    e2 = (0.5 * (es.astype(np.longdouble) ** 2)[None, :] + 0.5 * (et[at].astype(np.longdouble) ** 2)[:, None]
+          if kind == "symmetrized" else np.longdouble(0.01) ** 2)
+    want, mag = _reference(pos, tgt[at], idx[at], e2)
+    d = [torch.from_numpy(a).cuda() for a in (pos, tgt, idx.astype(np.int64), es, et)]
+    out = torch.empty((nt, 4), device="cuda", dtype=torch.float64)
+    rc = (bh.direct_force_sym(d[0], d[3], d[1], d[4], d[2], out, 64) if kind == "symmetrized"
+          else bh.direct_force(d[0], d[1], d[2], 0.01, out, 64))
+    assert rc == 0
+    assert (np.abs(out[torch.from_numpy(at).cuda()].cpu().numpy().astype(np.longdouble) - want) <= TOL[64] * mag).all()

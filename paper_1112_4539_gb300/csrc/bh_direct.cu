@@ -283,13 +283,16 @@ int launch_direct(const float4* src, int n_src, const float4* tgt, const int64_t
     };
     const int most = n_src / (4 * kDirThreads) + (n_src % (4 * kDirThreads) != 0);
     plan(kDirThreads, most);
-    // FP64 with less than two such blocks per SM: 32 targets per block, in as
-    // many partial sums as above, or 16 (which the shorter plain sums make up
-    // for), of a tile of sources at least.  Microseconds with 256 targets per
-    // block | 32: 1000 targets x 4000 sources 1073 | 162.  Error against FP64
-    // sums by PyTorch: 1.3e-16 at 256 x 1024 (2.8e-16 before), 1.4e-16
-    // (1.6e-16) at 256 x 2^14, 3.3e-16 (4.6e-16) at 256 x 2^18.
-    const bool narrow = precision == 64 && (long long)tblocks * split < 2 * sms;
+    // FP64 where such blocks leave an eighth or more of their waves empty: 32
+    // targets per block, in as many partial sums as above, or 16 (which the
+    // shorter plain sums make up for), of a tile of sources at least.
+    // Microseconds with 256 targets per block | 32, targets x sources: 256 x
+    // 1024 1065 | 58, 1000 x 4000 1069 | 162, 256 x 2^18 (256 blocks) 2121 |
+    // 1952, 1500 x 50000 (294 blocks, two full waves) 2119 | 2225.  Error
+    // against FP64 sums by PyTorch: 1.3e-16 at 256 x 1024 (2.8e-16 before),
+    // 1.4e-16 (1.5e-16) at 256 x 2^14, 3.3e-16 (4.4e-16) at 256 x 2^18.
+    const long long blocks = (long long)tblocks * split, waves = (blocks + sms - 1) / sms;
+    const bool narrow = precision == 64 && 9 * blocks < 8 * waves * sms;
     if (narrow) plan(32, max(most, min(16, n_src / kDirThreads + (n_src % kDirThreads != 0))));
     const int chunk = ((n_src + split - 1) / split + kDirThreads - 1) / kDirThreads * kDirThreads;
     split = max(1, (n_src + chunk - 1) / max(chunk, 1));

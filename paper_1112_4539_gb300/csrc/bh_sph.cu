@@ -33,6 +33,9 @@
 namespace bh {
 
 constexpr int kSphStackCap = kStackCap;  // ranges of <= 8 siblings; same bound as the gravity walk
+#ifndef BH_SPH_TEAM_STACK
+#define BH_SPH_TEAM_STACK kSphStackCap   // smaller only to see a block of warps report an overflow
+#endif
 constexpr int kSphRing = 64;             // candidates per ring (two tiles of 32)
 
 // ------------------------------------------------------------ node boxes
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
     bh_let_next_start();
     bh_after_previous();
     __shared__ SphSmem smem[NW == 1 ? 4 : NW];
-    __shared__ int s_group;
+    __shared__ int s_group, s_dead;  // NW > 1: the block's group; a warp's stack has overflowed
     __shared__ float s_rho[NW == 1 ? 1 : NW * T * 32];
     __shared__ int s_cnt[NW == 1 ? 1 : NW * T * 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -178,6 +181,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
     const int n_roots = (int)ctrl->level_offset[1];
     const int split = (int)ctrl->level_offset[kSphSplit], below = (int)ctrl->level_offset[kSphSplit + 1];
     unsigned long long tested = 0ull;
+    if (NW > 1 && threadIdx.x == 0) s_dead = 0;
 
     for (;;) {
         int g = 0;
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 leaf = leaf && ((keep >> at) & 1u);
             }
             const unsigned int om = __ballot_sync(BH_FULL_MASK, opn);
-            if (sp + __popc(om) > kSphStackCap) {
+            if (sp + __popc(om) > (NW == 1 ? kSphStackCap : BH_SPH_TEAM_STACK)) {
                 overflow = true;
                 break;
             }
@@ -364,9 +368,14 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 __syncwarp();
             }
         }
+        // (a block's warps leave together, after the barrier below: those left
+        // behind would wait for a group from the warp that has gone)
         if (overflow) {
-            if (lane == 0) bh_set_error(ctrl, BH_ERR_CAPACITY);
-            break;
+            if (lane == 0) {
+                bh_set_error(ctrl, BH_ERR_CAPACITY);
+                if (NW > 1) s_dead = 1;
+            }
+            if (NW == 1) break;
         }
         if (heavy) {
             if (lane == 0) P.heavy[atomicAdd(&ctrl->tile_ctr[0], 1u)] = g;
@@ -395,6 +404,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 s_rho[(wib * T + t) * 32 + lane] = rho[t];
             }
             __syncthreads();
+            if (s_dead) break;
             for (int t = wib; t < T; t += NW) {
                 int c = 0;
                 float d = 0.0f;

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "bh_mlp.cuh"
+#include "bh_wait.h"
 
 namespace bh {
 
@@ -457,9 +458,6 @@ struct WsTile {  // kTile sources as pairs, laid out as WarpSmem (points: a, b) 
 };
 
 // ------------------------------------------------------------ bounded mbarrier waits
-constexpr int kWsSpinLimit = 1 << 22;
-constexpr unsigned long long kWsTimeoutNs = 1000000000ull;
-
 __device__ __forceinline__ unsigned int bh_smem_addr(const void* p)
 {
     return static_cast<unsigned int>(__cvta_generic_to_shared(p));
@@ -484,7 +482,7 @@ __device__ __forceinline__ bool bh_mbar_try_wait(unsigned long long* b, unsigned
     return ok != 0u;
 }
 // Wait for the phase of the given parity to complete.  False (with the error
-// recorded) once a second has passed on the global timer or after
+// recorded) after a second of running time (WaitClock) or after
 // kWsSpinLimit polls, whichever comes first; false at once when another warp
 // has aborted.
 __device__ __forceinline__ unsigned long long bh_globaltimer()
@@ -496,12 +494,12 @@ __device__ __forceinline__ unsigned long long bh_globaltimer()
 __device__ __forceinline__ bool bh_mbar_wait(unsigned long long* b, unsigned int parity, bh_dev_ctrl* c)
 {
     if (bh_mbar_try_wait(b, parity)) return true;
-    const unsigned long long t0 = bh_globaltimer();
+    WaitClock t(bh_globaltimer());
     for (int i = 0; i < kWsSpinLimit; i++) {
         if (bh_mbar_try_wait(b, parity)) return true;
         if ((i & 63) == 63) {
             if (*(volatile unsigned int*)&c->abort) return false;
-            if (bh_globaltimer() - t0 > kWsTimeoutNs) break;
+            if (t.over(bh_globaltimer())) break;
         }
     }
     bh_set_error(c, BH_ERR_DEVICE_TIMEOUT);

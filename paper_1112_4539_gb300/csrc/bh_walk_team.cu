@@ -51,13 +51,13 @@ struct TileSum {
 __device__ __forceinline__ bool bh_turn_wait(const volatile int* turn, int i, bh_dev_ctrl* c)
 {
     if (*turn == i) return true;
-    const unsigned long long t0 = bh_globaltimer();
+    WaitClock t(bh_globaltimer());
     for (int k = 0; k < kWsSpinLimit; k++) {
         if (*turn == i) return true;
         __nanosleep(20);
         if ((k & 63) == 63) {
             if (*(volatile unsigned int*)&c->abort) return false;
-            if (bh_globaltimer() - t0 > kWsTimeoutNs) break;
+            if (t.over(bh_globaltimer())) break;
         }
     }
     bh_set_error(c, BH_ERR_DEVICE_TIMEOUT);

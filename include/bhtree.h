@@ -140,7 +140,8 @@ int tree_build(bh_ctx* ctx, const float* d_pos_mass, int64_t n, void* stream);
  * quadrupole second moment when the context's order is 2, and Eq. (2)'s
  * effective size S_eff = (l/theta + s)^2 (l = cube side, s = distance from
  * the cube centre to the centre of mass).  theta > 0.
- * Errors: BH_ERR_INVALID (theta <= 0 or not finite), BH_ERR_STATE (no tree). */
+ * Errors: BH_ERR_INVALID (theta <= 0 or not finite), BH_ERR_STATE (no tree, or
+ * the last one is bh_force_batched's, which computes its own moments). */
 int tree_moments(bh_ctx* ctx, float theta, void* stream);
 
 /* Step 5 of Sec. 4.4: the tree walk and force evaluation.  Each group of
@@ -272,7 +273,9 @@ int bh_batch_layout(bh_ctx* ctx, const int64_t* h_offsets, int nsys);
  * (ax, ay, az, phi) in the same order; systems never interact.  Same method
  * as tree_build + tree_moments(theta) + tree_force(eps) per system (plain
  * Eq. 2 criterion).  Stream-ordered, allocates nothing, syncs nothing: it can
- * be captured in a CUDA graph (see bh_graph_capture_batched).
+ * be captured in a CUDA graph (see bh_graph_capture_batched).  The context's tree
+ * is then that of all the systems: tree_moments, and with it tree_force and
+ * tree_force_particles, need a tree_build first.
  * Errors: BH_ERR_INVALID, BH_ERR_STATE (no layout, or the learned criterion is on). */
 int bh_force_batched(bh_ctx* ctx, const float* d_pos_mass, float theta, float eps, float* d_acc_pot, void* stream);
 

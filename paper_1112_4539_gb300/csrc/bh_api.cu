@@ -24,6 +24,7 @@ struct bh_ctx {
     bool deep = false;  // 63-bit keys (21 levels) instead of 30-bit keys (10 levels)
     int64_t n = -1;  // particles of the last tree_build (-1: none)
     bool have_moments = false;
+    bool batched = false;           // the last tree is bh_force_batched's
     float theta = 0.f;
     int64_t launches = 0;
     void* slab = nullptr;
@@ -319,6 +320,7 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
     x->launches += 1;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
+    x->batched = false;
     x->have_moments = false;
     x->have_soft = false;
     return BH_OK;
@@ -357,7 +359,9 @@ int tree_moments(bh_ctx* x, float theta, void* stream)
 {
     if (!x) return BH_ERR_INVALID;
     if (!(theta > 0.0f) || !std::isfinite(theta)) return BH_ERR_INVALID;
-    if (x->n < 0) return BH_ERR_STATE;
+    // a tree of several systems has no single root: S_eff needs each system's
+    // cube, and the per-particle walk starts at node 0
+    if (x->n < 0 || x->batched) return BH_ERR_STATE;
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
     if (x->n > 0) {
@@ -769,7 +773,8 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;
     x->theta = theta;
-    x->have_moments = false;  // the tree of several systems is not for tree_force
+    x->batched = true;        // the tree of several systems is not for tree_moments and the walks
+    x->have_moments = false;
     return BH_OK;
 }
 

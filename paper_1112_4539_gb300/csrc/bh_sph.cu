@@ -120,7 +120,7 @@ __device__ __forceinline__ float bh_w3(float r, float hinv, float c)
 
 // np pairs of candidates against the lane's targets; (nx, ny, nz): minus the
 // target, held twice.  The target itself is among the candidates once, at r2 =
-// 0 (the caller starts its count at -1).
+// 0 (the caller starts its count at -1), unless it has no finite place.
 template <int T>
 __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const float4* __restrict__ rb, int np,
                                             const f2 (&nx)[T], const f2 (&ny)[T], const f2 (&nz)[T],
@@ -229,9 +229,11 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
             hinv[t] = 1.0f / h;
             cw[t] = 8.0f / (3.14159265358979f * h * h * h);
             nx[t] = make_float2(-q.x, -q.x); ny[t] = make_float2(-q.y, -q.y); nz[t] = make_float2(-q.z, -q.z);
-            // the target's own pair has r2 = 0, below h^2 unless that underflows
+            // the target's own pair has r2 = 0, below h^2 unless that underflows;
+            // NaN for a coordinate that is no finite number, which has no neighbours
             const bool own = h2[t] > 0.0f, first = NW == 1 || wib == 0;
-            cnt[t] = own && first ? -1 : 0;
+            const bool finite = isfinite(q.x) && isfinite(q.y) && isfinite(q.z);
+            cnt[t] = own && first && finite ? -1 : 0;
             rho[t] = own || !first ? 0.0f : q.w * bh_w3(0.0f, hinv[t], cw[t]);
         }
         if (__any_sync(BH_FULL_MASK, bad)) {

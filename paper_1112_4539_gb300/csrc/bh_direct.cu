@@ -51,7 +51,8 @@ __device__ __forceinline__ void bh_kahan_r(R& s, R& c, R v)
 // is the other fma.  Error at most 1.25 2^-53, rms 0.46 2^-53 (4 million x over
 // all exponents on the host, any y0 within its bound; an FP64 third-order step
 // from a 20-bit estimate, 5 FP64 instructions, has 1.50 and 0.48).
-// Zero and denormal x give inf, inf gives 0.
+// Denormal x (no two FP32 places are that close: eps^2 alone) are scaled to
+// normal numbers and take two Newton steps; zero gives inf, inf gives 0.
 __device__ __forceinline__ double bh_rsqrt64(double x)
 {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
@@ -78,9 +79,12 @@ __device__ __forceinline__ double bh_rsqrt64(double x)
     const double r = __fma_rn(__hiloint2double((int)(h - 0x100000u), (int)(yb << 29)), d,
                               __hiloint2double((int)h, (int)((yb << 29) + ym)));
     if (hi - 0x100000u < 0x7fe00000u) return r;  // a normal number
+    const double s = x * 0x1p128;
     double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    return y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    if (x > 0.0 && hi < 0x100000u)
+        for (int i = 0; i < 2; i++) y = __fma_rn(0.5 * y, __fma_rn(-s * y, y, 1.0), y);
+    return y * 0x1p64;
 }
 
 // NARROW: a block takes 32 targets, one per lane, and its warps share each tile

@@ -92,3 +92,17 @@ def test_wide(n, nt, kind):
           else bh.direct_force(d[0], d[1], d[2], 0.01, out, 64))
     assert rc == 0
     assert (np.abs(out[torch.from_numpy(at).cuda()].cpu().numpy().astype(np.longdouble) - want) <= TOL[64] * mag).all()
+
+
+@pytest.mark.parametrize("eps", [2e-162, 1e-160, 3.3e-157, 1e-155, 1.49e-154, 1.5e-154])
+@pytest.mark.parametrize("nt", [1, 600])
+def test_denormal_softening(eps, nt):
+    """FP64, a source on the target: eps^2 is a denormal (a normal number from 1.4917e-154 on), its root within
+    2 units of 2^-53 and the product with the mass 1 more."""
+    import paper_1112_4539_gb300 as bh
+    src = torch.tensor([[0.5, -1.0, 2.0, 3.0]], device="cuda")
+    tgt = src.repeat(nt, 1).contiguous()
+    out = torch.empty((nt, 4), device="cuda", dtype=torch.float64)
+    assert bh.direct_force(src, tgt, None, eps, out, 64) == 0
+    want = -3.0 / np.sqrt(np.longdouble(np.float64(eps) * np.float64(eps)))
+    assert (np.abs(out[:, 3].cpu().numpy().astype(np.longdouble) / want - 1) <= 4 * 2.0 ** -53).all()

@@ -225,6 +225,9 @@ int tree_neighbors(bh_ctx* ctx, const float* d_h, float h, int32_t* d_count, flo
  * d_src: n_src float4 (x, y, z, m); d_tgt: n_tgt float4 (x, y, z, ignored).
  * precision 32: FP32 interactions, Kahan-compensated, d_out = n_tgt float4;
  * precision 64: FP64 throughout, d_out = n_tgt double4 (the error judge).
+ * Up to 1024 sources the sums are the same bits on every run; with more, few
+ * targets share the sources among blocks, whose partial sums are added as they
+ * come, and the last bits may differ.
  * No context is needed; nothing is allocated.
  * Errors: BH_ERR_INVALID (bad pointer/alignment/precision, eps < 0),
  * BH_ERR_TOO_LARGE (n_src or n_tgt >= 2^31). */

@@ -5,7 +5,9 @@
 // tile, Kahan-compensated across tiles.  FP64: the error judge, double
 // throughout.  When there are too few targets to fill the GPU the source range
 // is split across blocks and partial sums are combined with atomic adds into
-// the (zeroed) output.  The self term of each target is skipped by index, in
+// the (zeroed) output, so that their last bits depend on the order in which the
+// blocks end; up to 1024 sources the sums are the same bits on every run (one
+// block, or a cluster of up to four whose sums are added in order).  The self term of each target is skipped by index, in
 // the one tile that holds it.  With individual softening lengths (SYM) a pair
 // softens with (eps_i^2 + eps_j^2)/2, the symmetrized Plummer potential
 // (Sec. 7, after Saitoh & Makino 2010).
@@ -87,10 +89,26 @@ __device__ __forceinline__ double bh_rsqrt64(double x)
     return y * 0x1p64;
 }
 
+// Sums of targets held in a block's shared memory, v[32], read by another block of its cluster.
+__device__ __forceinline__ bh_double4 bh_cluster_read(const bh_double4* v, unsigned int rank)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;"
+        : "=r"(at)
+        : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(v))), "r"(rank));
+    bh_double4 r;
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "r"(at) : "memory");
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(r.z), "=d"(r.w) : "r"(at + 16) : "memory");
+    return r;
+}
+
+// How the blocks of one target put their sums together.
+enum class Join { one, atomic, cluster };  // a single block | atomic adds | in order (NARROW only)
+
 // NARROW: a block takes 32 targets, one per lane, and its warps share each tile
 // of sources, 32 each; their sums are put together at the end with their
 // compensations.
-template <bool NARROW, bool ATOMIC, bool SYM>
+template <bool NARROW, Join JOIN, bool SYM>
 __global__ void __launch_bounds__(kDirThreads)
 bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __restrict__ tgt,
                    const int64_t* __restrict__ self, int n_tgt, double eps2, bh_double4* __restrict__ out, int chunk,
@@ -161,19 +179,32 @@ bh_direct64_kernel(const float4* __restrict__ src, int n_src, const float4* __re
         tile[threadIdx.x] = bh_double4{ax, ay, az, ph};
         rest[threadIdx.x] = bh_double4{cx, cy, cz, cp};
         __syncthreads();
-        if (first != 0 || !valid) return;
-        for (int k = lane + 32; k < kDirThreads; k += 32) {
-            const bh_double4 v = tile[k], c = rest[k];
+        auto add = [&](bh_double4 v, bh_double4 c) {
             cx += c.x; cy += c.y; cz += c.z; cp += c.w;
             bh_kahan_r<double>(ax, cx, v.x);
             bh_kahan_r<double>(ay, cy, v.y);
             bh_kahan_r<double>(az, cz, v.z);
             bh_kahan_r<double>(ph, cp, v.w);
+        };
+        if (first == 0)
+            for (int k = lane + 32; k < kDirThreads; k += 32) add(tile[k], rest[k]);
+        if (JOIN == Join::cluster) {
+            if (first == 0) {
+                tile[lane] = bh_double4{ax, ay, az, ph};
+                rest[lane] = bh_double4{cx, cy, cz, cp};
+            }
+            bh_cluster_sync();
+            if (first == 0 && blockIdx.y == 0)
+                for (unsigned int b = 1; b < gridDim.y; b++)
+                    add(bh_cluster_read(tile + lane, b), bh_cluster_read(rest + lane, b));
+            bh_cluster_sync();  // (a block's shared memory lasts until it is read)
+            if (blockIdx.y != 0) return;
         }
+        if (first != 0) return;
     }
     if (!valid) return;
     const double rx = ax - cx, ry = ay - cy, rz = az - cz, rp = ph - cp;
-    if (ATOMIC) {
+    if (JOIN == Join::atomic) {
         double* o = reinterpret_cast<double*>(out + i);
         atomicAdd(o + 0, rx);
         atomicAdd(o + 1, ry);
@@ -302,11 +333,22 @@ int launch_direct(const float4* src, int n_src, const float4* tgt, const int64_t
     split = max(1, (n_src + chunk - 1) / max(chunk, 1));
     const dim3 grid(tblocks, split);
     const size_t rec = precision == 64 ? sizeof(bh_double4) : sizeof(float4);
-    if (split > 1 || n_src == 0) cudaMemsetAsync(out, 0, (size_t)n_tgt * rec, s);
+    // few sources gave one block per target, hence the same bits on every run: they keep them
+    const bool in_order = narrow && most == 1 && split > 1;
+    if ((split > 1 && !in_order) || n_src == 0) cudaMemsetAsync(out, 0, (size_t)n_tgt * rec, s);
     if (n_src == 0) return BH_OK;
     auto launch64 = [&](auto kern) {
-        kern<<<grid, kDirThreads, 0, s>>>(src, n_src, tgt, self, n_tgt, sym ? 0.0 : eps * eps, (bh_double4*)out, chunk,
-                                          eps_src, eps_tgt);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {1u, (unsigned int)(in_order ? split : 1), 1u};
+        cudaLaunchConfig_t c = {};
+        c.gridDim = grid;
+        c.blockDim = kDirThreads;
+        c.stream = s;
+        c.attrs = at;
+        c.numAttrs = in_order ? 1 : 0;
+        cudaLaunchKernelEx(&c, kern, src, n_src, tgt, self, n_tgt, sym ? 0.0 : eps * eps, (bh_double4*)out, chunk,
+                           eps_src, eps_tgt);
     };
     auto launch32 = [&](auto kern) {
         kern<<<grid, kDirThreads, 0, s>>>(src, n_src, tgt, self, n_tgt, sym ? 0.0f : (float)(eps * eps), (float4*)out,
@@ -314,13 +356,17 @@ int launch_direct(const float4* src, int n_src, const float4* tgt, const int64_t
     };
     const bool at = split > 1, normal = !sym && (float)(eps * eps) >= 1.17549435e-38f;
     if (precision == 64) {
-        auto choose = [&](auto form) {
+        auto choose = [&](auto form, auto join) {
             constexpr bool N = decltype(form)::value;
-            if (sym) at ? launch64(bh_direct64_kernel<N, true, true>) : launch64(bh_direct64_kernel<N, false, true>);
-            else at ? launch64(bh_direct64_kernel<N, true, false>) : launch64(bh_direct64_kernel<N, false, false>);
+            constexpr Join J = decltype(join)::value;
+            sym ? launch64(bh_direct64_kernel<N, J, true>) : launch64(bh_direct64_kernel<N, J, false>);
         };
-        if (narrow) choose(std::true_type());
-        else choose(std::false_type());
+        using One = std::integral_constant<Join, Join::one>;
+        using Atomic = std::integral_constant<Join, Join::atomic>;
+        using Cluster = std::integral_constant<Join, Join::cluster>;
+        if (in_order) choose(std::true_type(), Cluster());
+        else if (narrow) at ? choose(std::true_type(), Atomic()) : choose(std::true_type(), One());
+        else at ? choose(std::false_type(), Atomic()) : choose(std::false_type(), One());
     } else if (sym) {
         at ? launch32(bh_direct32_kernel<true, true, false>) : launch32(bh_direct32_kernel<false, true, false>);
     } else if (normal) {

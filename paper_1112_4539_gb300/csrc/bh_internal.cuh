@@ -286,6 +286,12 @@ __device__ __forceinline__ unsigned int bh_match_digit(unsigned int d, bool ok)
     return peers;
 }
 
+// Barrier of all threads of a cluster; what each wrote before it is visible to all after it.
+__device__ __forceinline__ void bh_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 __device__ __forceinline__ int bh_warp_incl_scan(int v)
 {
     const int lane = threadIdx.x & 31;

@@ -106,3 +106,25 @@ def test_denormal_softening(eps, nt):
     assert bh.direct_force(src, tgt, None, eps, out, 64) == 0
     want = -3.0 / np.sqrt(np.longdouble(np.float64(eps) * np.float64(eps)))
     assert (np.abs(out[:, 3].cpu().numpy().astype(np.longdouble) / want - 1) <= 4 * 2.0 ** -53).all()
+
+
+@pytest.mark.parametrize("n,nt", [(257, 1), (600, 33), (1000, 9000), (1024, 256), (1024, 40000)])
+@pytest.mark.parametrize("kind", ["softened", "symmetrized"])
+def test_few_sources_repeat(n, nt, kind):
+    """FP64, up to 1024 sources (two to four partial sums per target): the same bits on every run."""
+    import paper_1112_4539_gb300 as bh
+    src, tgt = torch.from_numpy(workloads.plummer(n, seed=n)).cuda(), torch.from_numpy(workloads.plummer(nt, seed=98)).cuda()
+    es, et = (torch.from_numpy(workloads.softening_lengths(k, 0.01)).cuda() for k in (n, nt))
+    busy, out = torch.empty(1 << 22, device="cuda"), torch.empty((60, nt, 4), device="cuda", dtype=torch.float64)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for k in range(60):
+        if k % 2:
+            with torch.cuda.stream(side):  # (the blocks end in another order beside other work)
+                busy.mul_(1.0)
+        out[k].fill_(float(k))
+        rc = (bh.direct_force_sym(src, es, tgt, et, None, out[k], 64) if kind == "symmetrized"
+              else bh.direct_force(src, tgt, None, 0.01, out[k], 64))
+        assert rc == 0
+    torch.cuda.synchronize()
+    assert (out == out[0]).all()

@@ -429,7 +429,7 @@ int tree_neighbors(bh_ctx* x, const float* d_h, float h, int32_t* d_count, float
     if (d_rho && (((uintptr_t)d_rho & 3u) || !is_device_ptr(d_rho, x->device))) return BH_ERR_INVALID;
     DeviceGuard guard(x->device);
     int rc = bh::launch_sph(x->pos_s, x->vals, x->g_first, x->g_count, x->nd, x->blo, x->bhi, x->cfg.group_size, d_h,
-                            h, d_count, d_rho, (int32_t*)x->vals_alt, x->ctrl, x->sm_count, grid_for(x), x->cfg.max_level,
+                            h, d_count, d_rho, (int32_t*)x->vals_alt, (int)x->n, x->ctrl, x->sm_count, grid_for(x), x->cfg.max_level,
                             (cudaStream_t)stream);
     if (rc) return rc;
     x->launches += bh::launches_sph(x->deep);

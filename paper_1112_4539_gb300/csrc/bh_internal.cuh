@@ -51,7 +51,9 @@ struct bh_dev_ctrl {
     unsigned int scan_done;      // level-scan blocks finished (the last one writes the offsets)
     unsigned int cost_count[16]; // groups of each cost class (bh_group_order_kernel)
     unsigned int cost_taken[16];
-    unsigned int pad[6];
+    unsigned long long sph_like; // neighbour search: candidates that its sample of groups expects
+    unsigned int sph_samples;
+    unsigned int pad[3];
 };
 
 // Record a device-side error (first one wins) and raise the abort flag.
@@ -467,13 +469,13 @@ void launch_softening(const float* eps, const uint32_t* perm, const float4* pos_
 
 int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                const bh_nodes& nd, float4* blo, float4* bhi, int G, const float* h, float h_const, int32_t* count,
-               float* rho, int32_t* heavy, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
+               float* rho, int32_t* heavy, int n, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s);
 
 // launches per call (deep = 63-bit keys: 8 sort passes, 22 levels)
 inline int launches_build(bool deep) { return deep ? 19 : 15; }  // init, bbox, keys, sort passes, 4 tree, 4 groups
 constexpr int kLaunchesForce = 2;    // counter reset, walk
 constexpr int kLaunchesPWalk = 4;    // parent links, next links, counter reset, walk
-inline int launches_sph(bool deep) { return (deep ? 22 : 11) + 3; }  // node boxes per level, reset, two walks
+inline int launches_sph(bool deep) { return (deep ? 22 : 11) + 2; }  // node boxes per level, two walks
 inline int launches_softening(bool deep) { return (deep ? 22 : 11) + 1; }  // gather, one per level
 
 }  // namespace bh

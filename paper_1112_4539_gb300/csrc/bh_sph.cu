@@ -38,16 +38,77 @@ constexpr int kSphStackCap = kStackCap;  // ranges of <= 8 siblings; same bound 
 #endif
 constexpr int kSphRing = 64;             // candidates per ring (two tiles of 32)
 
+struct SphParams {
+    const float4* pos_s;
+    const uint32_t* perm;
+    const int32_t* g_first;
+    const int32_t* g_count;
+    const int4* rec;
+    const float4* blo;
+    const float4* bhi;
+    const float* h;      // per particle, caller order (nullptr: h_const)
+    float h_const;
+    int32_t* count;      // caller order (nullptr: not written)
+    float* rho;          // caller order (nullptr: not written)
+    bh_dev_ctrl* ctrl;
+    int32_t* heavy;      // groups left to the second launch (tile_ctr[0] of them)
+    int max_level;
+};
+
+// What a group at large costs: candidates at the density of its box, n at most,
+// added up over 1024 groups spread over the list (whole numbers, so that the sum
+// is the same in any order).  Groups of few particles say little about their density.
+constexpr int kSphSamples = 1024;
+constexpr int kSphSampleLevel = 6;  // (the deepest is 10 or 21)
+__device__ __forceinline__ void bh_sph_sample(const SphParams& P, int n)
+{
+    const int lane = threadIdx.x & 31, ng = (int)P.ctrl->n_groups;
+    if (ng <= kSphSamples) return;
+    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < kSphSamples; w += (gridDim.x * blockDim.x) >> 5) {
+        const int g = (int)((long long)ng * w / kSphSamples), gb = P.g_first[g], gc = P.g_count[g];
+        if (gc < 8) continue;
+        float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, h = 0.0f;
+        for (int o = lane; o < gc; o += 32) {
+            const float4 q = P.pos_s[gb + o];
+            h = fmaxf(h, P.h ? P.h[P.perm[gb + o]] : P.h_const);
+            lo[0] = fminf(lo[0], q.x); lo[1] = fminf(lo[1], q.y); lo[2] = fminf(lo[2], q.z);
+            hi[0] = fmaxf(hi[0], q.x); hi[1] = fmaxf(hi[1], q.y); hi[2] = fmaxf(hi[2], q.z);
+        }
+        h = bh_ord2f(__reduce_max_sync(BH_FULL_MASK, bh_f2ord(h)));
+        float side = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            side = fmaxf(side, bh_ord2f(__reduce_max_sync(BH_FULL_MASK, bh_f2ord(hi[k]))) -
+                                   bh_ord2f(__reduce_min_sync(BH_FULL_MASK, bh_f2ord(lo[k]))));
+        const float r = 1.0f + 2.0f * h / side;
+        if (lane == 0) {
+            atomicAdd(&P.ctrl->sph_like, (unsigned long long)fminf((float)gc * (r * r * r), (float)n));
+            atomicAdd(&P.ctrl->sph_samples, 1u);
+        }
+    }
+}
+
 // ------------------------------------------------------------ node boxes
 // Tight bounding box of every node's particles, bottom-up by level: a leaf
 // scans its particles, an internal node combines its children (one level
-// deeper, already done).  Min/max are exact.
+// deeper, already done).  Min/max are exact.  The first launch clears the search's
+// counters; that of a level with many nodes samples the groups beside them.
 __global__ void __launch_bounds__(256)
 bh_node_box_kernel(const float4* __restrict__ pos_s, const int4* __restrict__ rec, float4* __restrict__ lo,
-                   float4* __restrict__ hi, int lev, const bh_dev_ctrl* __restrict__ c)
+                   float4* __restrict__ hi, int lev, SphParams P, int n)
 {
     bh_let_next_start();
-    bh_after_previous(pos_s, rec, lo, hi, c);
+    bh_after_previous(pos_s, rec, lo, hi);
+    bh_dev_ctrl* c = P.ctrl;
+    if (lev == P.max_level && blockIdx.x == 0 && threadIdx.x == 0) {  // the search's counters
+        c->group_ctr = 0u;
+        c->tile_ctr[0] = 0u;  // groups listed as heavy (the sort's tickets are free after the build)
+        c->tile_ctr[1] = 0u;  // and taken
+        c->sph_like = 0ull;
+        c->sph_samples = 0u;
+        c->n_pp = 0ull;
+        c->n_pc = 0ull;
+    }
     const int v0 = (int)c->level_offset[lev], v1 = (int)c->level_offset[lev + 1];
     for (int v = v0 + blockIdx.x * blockDim.x + threadIdx.x; v < v1; v += gridDim.x * blockDim.x) {
         const int4 r = rec[v];
@@ -83,6 +144,7 @@ bh_node_box_kernel(const float4* __restrict__ pos_s, const int4* __restrict__ re
         lo[v] = a;
         hi[v] = b;
     }
+    if (lev == kSphSampleLevel) bh_sph_sample(P, n);
 }
 
 // ------------------------------------------------------------ walk
@@ -91,22 +153,6 @@ struct SphSmem {
     int2 leafq[32];
     float4 blo[32], bhi[32];                      // boxes of the pop's near leaves
     float4 ra[kSphRing / 2], rb[kSphRing / 2];    // candidates as pairs: (x, x', y, y') (z, z', m, m')
-};
-
-struct SphParams {
-    const float4* pos_s;
-    const uint32_t* perm;
-    const int32_t* g_first;
-    const int32_t* g_count;
-    const int4* rec;
-    const float4* blo;
-    const float4* bhi;
-    const float* h;      // per particle, caller order (nullptr: h_const)
-    float h_const;
-    int32_t* count;      // caller order (nullptr: not written)
-    float* rho;          // caller order (nullptr: not written)
-    bh_dev_ctrl* ctrl;
-    int32_t* heavy;      // groups left to the second launch (tile_ctr[0] of them)
 };
 
 // cubic spline with support h (normalised to unit integral), FP32
@@ -120,7 +166,8 @@ __device__ __forceinline__ float bh_w3(float r, float hinv, float c)
 
 // np pairs of candidates against the lane's targets; (nx, ny, nz): minus the
 // target, held twice.  The target itself is among the candidates once, at r2 =
-// 0 (the caller starts its count at -1), unless it has no finite place.
+// 0 (the caller starts its count at -1); one without a finite place has no pair,
+// not even its own, and its count of -1 is written as 0.
 template <int T>
 __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const float4* __restrict__ rb, int np,
                                             const f2 (&nx)[T], const f2 (&ny)[T], const f2 (&nz)[T],
@@ -148,12 +195,23 @@ __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const
     }
 }
 
-// NW = 1: a warp per group, which gives up a group after kSphHeavy candidates or
-// kSphPops batches of nodes and lists it.  NW > 1: a block of NW warps per
+// NW = 1: a warp per group, which gives up a group after `most` candidates or one
+// batch of nodes per 16 of them and lists it.  NW > 1: a block of NW warps per
 // listed group, which share its subtrees; their counts and densities are added
 // in warp order.  A group's work varies with its radii (in a Plummer sphere's
 // outskirts the radius that holds 64 neighbours reaches into the core), and the
 // few long ones were the whole tail of the launch.
+//
+// A listed group is walked again from the start, so the limit must leave alone
+// what is no exception.  While every warp has a group at most, idle warps are
+// plenty and it is kSphHeavy; with more groups it is at least twice what a
+// group at large costs (bh_sph_sample), and a quarter of a warp's share.  All of
+// this is the same on every run, and so are the densities' bits.  The block's
+// warps share the subtrees of about half the search radius: from one level
+// (4) on a dense knot's neighbourhood was a single subtree, of one warp.
+// ms, start of both | 1024 throughout, level 4 | this: clumpy 2^20, 500
+// neighbours, G = 32 6.96 | 17.2 | 5.5, 32 neighbours 2.01 | 3.20 | 1.5; uniform
+// 2^20, 500, G = 64 3.80 | 5.28 | 3.1; Plummer 250000, 32, G = 64 10.5 | 2.16 | 2.17.
 //
 // GB300, build and search, a warp per group throughout -> this (the same counts):
 // Plummer 131072, G = 32 1.56 -> 0.77 ms, 4000 particles 580 -> 477 us, 2^20
@@ -161,7 +219,7 @@ __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const
 // 0.72 / 0.77 / 0.90 ms; of 512 / 1024 / 2048 candidates at 2^20 1.17 / 1.10 / 1.10.
 constexpr int kSphHeavy = 1024;
 constexpr int kSphPops = 64;
-constexpr int kSphSplit = 4;  // the level whose subtrees are shared out
+constexpr int kSphSplit = 4;  // the least level whose subtrees are shared out
 template <int T>
 constexpr int bh_sph_team() { return T <= 3 ? 8 : 4; }  // (shared memory)
 template <int T, int NW>
@@ -170,7 +228,8 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
     bh_let_next_start();
     bh_after_previous();
     __shared__ SphSmem smem[NW == 1 ? 4 : NW];
-    __shared__ int s_group, s_dead;  // NW > 1: the block's group; a warp's stack has overflowed
+    __shared__ int s_group;
+    __shared__ volatile int s_most;  // NW = 1: candidates after which a group is given up (volatile: in no register)
     __shared__ float s_rho[NW == 1 ? 1 : NW * T * 32];
     __shared__ int s_cnt[NW == 1 ? 1 : NW * T * 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -179,9 +238,17 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
     bh_dev_ctrl* ctrl = P.ctrl;
     const int ng = (int)ctrl->n_groups;
     const int n_roots = (int)ctrl->level_offset[1];
-    const int split = (int)ctrl->level_offset[kSphSplit], below = (int)ctrl->level_offset[kSphSplit + 1];
     unsigned long long tested = 0ull;
-    if (NW > 1 && threadIdx.x == 0) s_dead = 0;
+    if (NW == 1) {
+        if (threadIdx.x == 0) {
+            const float load = (float)ng / (4.0f * (float)gridDim.x);  // groups per warp
+            float most = (float)kSphHeavy;
+            if (load > 1.0f && ctrl->sph_samples)
+                most = fmaxf(most, fmaxf(2.0f, 0.25f * load) * ((float)ctrl->sph_like / (float)ctrl->sph_samples));
+            s_most = (int)fminf(most, 1e9f);
+        }
+        __syncthreads();
+    }
 
     for (;;) {
         int g = 0;
@@ -229,11 +296,9 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
             hinv[t] = 1.0f / h;
             cw[t] = 8.0f / (3.14159265358979f * h * h * h);
             nx[t] = make_float2(-q.x, -q.x); ny[t] = make_float2(-q.y, -q.y); nz[t] = make_float2(-q.z, -q.z);
-            // the target's own pair has r2 = 0, below h^2 unless that underflows;
-            // NaN for a coordinate that is no finite number, which has no neighbours
+            // the target's own pair has r2 = 0, below h^2 unless that underflows
             const bool own = h2[t] > 0.0f, first = NW == 1 || wib == 0;
-            const bool finite = isfinite(q.x) && isfinite(q.y) && isfinite(q.z);
-            cnt[t] = own && first && finite ? -1 : 0;
+            cnt[t] = own && first ? -1 : 0;
             rho[t] = own || !first ? 0.0f : q.w * bh_w3(0.0f, hinv[t], cw[t]);
         }
         if (__any_sync(BH_FULL_MASK, bad)) {
@@ -263,12 +328,19 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
             if (P.rec[mid].x <= gb) root = mid;
             else hi = mid;
         }
+        // NW > 1: the first node and the end of the level whose subtrees are shared out
+        int split = 0, below = 0;
+        if (NW > 1) {
+            const int lev = ilogbf(fminf(fmaxf(ctrl->box[3] / hmax, 1.0f), 1e9f)) + 1;
+            split = (int)ctrl->level_offset[max(kSphSplit, min(lev, P.max_level))];
+            below = (int)ctrl->level_offset[max(kSphSplit, min(lev, P.max_level)) + 1];
+        }
         int sp = 1, ring_head = 0, ring_cnt = 0, pops = 0, taken = 0;
         if (lane == 0) S.stack[0] = (uint32_t)root << 3;
         __syncwarp();
         bool overflow = false, heavy = false;
         while (sp > 0) {
-            if (NW == 1 && (taken >= kSphHeavy || pops++ >= kSphPops)) {
+            if (NW == 1 && max(taken, kSphHeavy / kSphPops * pops++) >= s_most) {
                 heavy = true;
                 break;
             }
@@ -292,7 +364,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 near = gx * gx + gy * gy + gz * gz <= reach2;
             }
             // a block's warps walk the top of the tree alike and share out its
-            // leaves and the subtrees from level kSphSplit down by node index
+            // leaves and the subtrees from the split level down by node index
             if (NW > 1 && v < below && (v >= split || r.z < 0)) near = near && v % NW == wib;
             bool leaf = near && r.z < 0;
             const bool opn = near && r.z >= 0;
@@ -370,13 +442,11 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 __syncwarp();
             }
         }
-        // (a block's warps leave together, after the barrier below: those left
-        // behind would wait for a group from the warp that has gone)
+        // (a block's warps leave together, at the next group, which thread 0 does
+        // not take once the error is set: if it left here, the others would find
+        // its last group for ever)
         if (overflow) {
-            if (lane == 0) {
-                bh_set_error(ctrl, BH_ERR_CAPACITY);
-                if (NW > 1) s_dead = 1;
-            }
+            if (lane == 0) bh_set_error(ctrl, BH_ERR_CAPACITY);
             if (NW == 1) break;
         }
         if (heavy) {
@@ -406,7 +476,6 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 s_rho[(wib * T + t) * 32 + lane] = rho[t];
             }
             __syncthreads();
-            if (s_dead) break;
             for (int t = wib; t < T; t += NW) {
                 int c = 0;
                 float d = 0.0f;
@@ -417,7 +486,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
                 const int o = t * 32 + lane;
                 if (o < gc) {
                     const uint32_t dst = P.perm[gb + o];
-                    if (P.count) P.count[dst] = c;
+                    if (P.count) P.count[dst] = max(c, 0);
                     if (P.rho) P.rho[dst] = d;
                 }
             }
@@ -428,7 +497,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
             const int o = t * 32 + lane;
             if (o < gc) {
                 const uint32_t dst = P.perm[gb + o];
-                if (P.count) P.count[dst] = cnt[t];
+                if (P.count) P.count[dst] = max(cnt[t], 0);
                 if (P.rho) P.rho[dst] = rho[t];
             }
         }
@@ -437,17 +506,6 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : NW * 32) bh_sph_kernel(SphPara
         atomicAdd(&ctrl->n_pp, tested);
         atomicAdd(&ctrl->cum_pp, tested);
     }
-}
-
-__global__ void bh_sph_reset_kernel(bh_dev_ctrl* c)
-{
-    bh_let_next_start();
-    bh_after_previous();
-    c->group_ctr = 0u;
-    c->tile_ctr[0] = 0u;  // groups listed as heavy (the sort's tickets are free after the build)
-    c->tile_ctr[1] = 0u;  // and taken
-    c->n_pp = 0ull;
-    c->n_pc = 0ull;
 }
 
 // persistent grid: as many blocks per SM as the registers and shared memory allow
@@ -472,11 +530,8 @@ static int bh_sph_launch(const SphParams& P, int sm_count, cudaStream_t s)
 
 int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                const bh_nodes& nd, float4* blo, float4* bhi, int G, const float* h, float h_const, int32_t* count,
-               float* rho, int32_t* heavy, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s)
+               float* rho, int32_t* heavy, int n, bh_dev_ctrl* ctrl, int sm_count, int grid, int max_level, cudaStream_t s)
 {
-    for (int lev = max_level; lev >= 0; lev--)
-        bh_launch_after(bh_node_box_kernel, grid, 256, 0, s, pos_s, nd.rec, blo, bhi, lev, ctrl);
-    bh_launch_after(bh_sph_reset_kernel, 1, 1, 0, s, ctrl);
     SphParams P;
     P.pos_s = pos_s;
     P.perm = perm;
@@ -491,6 +546,9 @@ int launch_sph(const float4* pos_s, const uint32_t* perm, const int32_t* g_first
     P.rho = rho;
     P.ctrl = ctrl;
     P.heavy = heavy;
+    P.max_level = max_level;
+    for (int lev = max_level; lev >= 0; lev--)
+        bh_launch_after(bh_node_box_kernel, grid, 256, 0, s, pos_s, nd.rec, blo, bhi, lev, P, n);
     const int T = G <= 32 ? 1 : G <= 64 ? 2 : G <= 96 ? 3 : G <= 128 ? 4 : 8;
     switch (T) {
         case 1: return bh_sph_launch<1>(P, sm_count, s);

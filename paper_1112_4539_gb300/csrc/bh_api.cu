@@ -47,6 +47,8 @@ struct bh_ctx {
     // several independent systems
     int nsys = 0;                   // systems of the current layout (0: none)
     int64_t batch_n = 0;            // their total particle count
+    int batch_filled = 0;           // systems with particles
+    double batch_groups = 0.0;      // about how many groups they have (bh::WalkSet)
     uint32_t* sys_of = nullptr;     // system of each Morton position
     int32_t* sys_off = nullptr;     // first particle of each system (+ total)
     float4* sys_box = nullptr;      // root cube of each system
@@ -391,7 +393,7 @@ int tree_force(bh_ctx* x, float eps, float* d_acc_pot, void* stream)
     bh::WalkLearned wl{x->mfeat, x->mlp, x->theta};
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count, x->cfg.block_threads,
-                             x->cfg.blocks_per_sm, (int)x->n, x->deep, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
+                             x->cfg.blocks_per_sm, bh::WalkSet((int)x->n, x->cfg.group_size), x->deep, s, x->mac_learned ? &wl : nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     x->launches += bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
@@ -724,11 +726,15 @@ int bh_batch_layout(bh_ctx* x, const int64_t* h_offsets, int nsys)
     if (nsys > x->cfg.max_systems) return BH_ERR_TOO_LARGE;
     if (h_offsets[0] != 0) return BH_ERR_INVALID;
     std::vector<int32_t> off32((size_t)nsys + 1);
+    int filled = 0;
+    double groups = 0.0;
     for (int s = 0; s < nsys; s++) {
         const int64_t c = h_offsets[s + 1] - h_offsets[s];
         if (c < 0) return BH_ERR_INVALID;
         if (c > bh::kBatchMaxN) return BH_ERR_TOO_LARGE;
         off32[(size_t)s] = (int32_t)h_offsets[s];
+        filled += c > 0;
+        groups += bh::WalkSet::of_system(c, x->cfg.group_size);
     }
     if (h_offsets[nsys] > x->max_n) return BH_ERR_TOO_LARGE;
     off32[(size_t)nsys] = (int32_t)h_offsets[nsys];
@@ -738,6 +744,8 @@ int bh_batch_layout(bh_ctx* x, const int64_t* h_offsets, int nsys)
         return BH_ERR_CUDA;
     x->nsys = nsys;
     x->batch_n = h_offsets[nsys];
+    x->batch_filled = filled;
+    x->batch_groups = groups;
     return BH_OK;
 }
 
@@ -764,7 +772,8 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
                        x->cfg.curve, N, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count,
-                             x->cfg.block_threads, x->cfg.blocks_per_sm, N, x->deep, s,
+                             x->cfg.block_threads, x->cfg.blocks_per_sm, bh::WalkSet(N, x->batch_filled, x->batch_groups),
+                             x->deep, s,
                              nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     // init, batch sort, 4 tree, 3 or 4 groups, moments per level, 2 walk

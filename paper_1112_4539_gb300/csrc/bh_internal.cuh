@@ -439,10 +439,55 @@ struct WalkLearned {
     const bh_mlp_dev* mlp;
     float theta_guard;
 };
+// What launch_walk is to expect: the particles, the systems they form (of a
+// batched call) and about how many groups: measured 0.65-0.75 G particles each, a
+// whole system where it is no larger than a group, and one more in every other.
+struct WalkSet {
+    int n, systems = 1;
+    double groups;
+    WalkSet(int n_, int G) : n(n_), groups(n_ / (0.65 * G)) {}
+    WalkSet(int n_, int systems_, double groups_) : n(n_), systems(systems_), groups(groups_) {}
+    static double of_system(long long n, int G) { return n <= 0 ? 0.0 : n <= G ? 1.0 : n / (0.65 * G) + 1.0; }
+};
+
+constexpr int kTeamMaxGroup = 128;  // targets per group that the team walk holds
+// Warps per group of the team walk (bh_walk_team.cu), 0: a warp per group
+// (bh_walk_kernel).  Eight while every group can have a block of its own at once
+// (two such blocks per SM; the walker, at about 1.5 us per 32 nodes, sets the pace), else
+// four (four blocks per SM, as many walkers again): clumpy 16384, G = 96, 183 us
+// with four and 147 with eight, Plummer 65536, G = 64, 657 and 694.
+// One launch, us, on GB300, groups taken by falling cost on both sides:
+//                                     one warp   block
+//   Plummer 4096, order 1, G = 64          166      75
+//   clumpy 16384, order 2, G = 96          468     125
+//   Plummer 70000, order 1, G = 64         798     470
+//   clumpy 100003, order 2, G = 96         679     540
+//   Plummer 150000, order 2, G = 96       1864    1079
+//   clumpy 150000, order 2, G = 96         830     729
+//   clumpy 200000, order 2, G = 128        904     977
+//   clumpy 100000, order 1, G = 64         283     320
+//   Plummer 120000, order 2, G = 32        505     656
+//   Plummer 262144, order 2, G = 96       1101    1428
+// From about one group per warp of bh_walk_kernel's grid on (16 warps per SM) the
+// groups fill the GPU by themselves and the walkers' idle issue slots cost more
+// than the split gains.  (Near the limit it depends on the set as well: a Plummer
+// sphere, whose walks are long, still gains, clumps or few terms lose up to 13%.)
+// Batched calls of systems of fewer than 2048 particles on average have short walks,
+// for which a block pays only while all groups have one at once.  Whole calls, us,
+// one warp | block, order 1: 256 systems of 256, G = 64 152 | 177, G = 96 155 | 166,
+// 64 of 256, G = 96 120 | 124, 32 of 256 117 | 107, 64 of 2048 303 | 315, 32 of 2048
+// 245 | 234, 16 of 8192 666 | 540, 5000 of 4 to 8 221 | 281.
+inline int bh_team_warps(const WalkSet& set, int G, int sm_count)
+{
+    const bool batch = set.systems > 1 && set.n < 2048.0 * set.systems;
+    if (G > kTeamMaxGroup || set.groups > (batch ? 2.0 : 16.0) * sm_count) return 0;
+    return set.groups <= 4.0 * sm_count ? 8 : 4;
+}
+
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl,
-                int sm_count, int block_threads, int blocks_per_sm, int n, bool deep, cudaStream_t s,
+                int sm_count, int block_threads, int blocks_per_sm, const WalkSet& set, bool deep, cudaStream_t s,
                 const WalkLearned* learned = nullptr, int walk_variant = 0);
 // failure-path self-tests: one bounded wait that nothing satisfies
 void launch_selftest_ring(bh_dev_ctrl* c, cudaStream_t s);

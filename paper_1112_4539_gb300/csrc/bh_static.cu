@@ -185,7 +185,7 @@ extern "C" int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh
     }
     bh::launch_moments(pos_s, keys, false, nd, c.order, theta, c.fp64_node_threshold, c.curve, N32, ctrl, grid, s);
     int rc = bh::launch_walk(pos_s, vals, g_first, g_count, (const int32_t*)keys_alt, nd, c.order, c.group_size, eps, (float4*)d_acc_pot, ctrl,
-                             sd.sm_count, c.block_threads, c.blocks_per_sm, N32, false, s, nullptr, c.walk_variant);
+                             sd.sm_count, c.block_threads, c.blocks_per_sm, bh::WalkSet(N32, c.group_size), false, s, nullptr, c.walk_variant);
     if (rc) return rc;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     if (h_status) {

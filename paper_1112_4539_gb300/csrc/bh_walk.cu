@@ -1264,7 +1264,8 @@ static int bh_walk_dispatch(const WalkParams& P, int order, int G, int sm_count,
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl, int sm_count,
-                int block_threads, int blocks_per_sm, int n, bool deep, cudaStream_t s, const WalkLearned* learned, int walk_variant)
+                int block_threads, int blocks_per_sm, const WalkSet& set, bool deep, cudaStream_t s,
+                const WalkLearned* learned, int walk_variant)
 {
     bh_launch_after(bh_walk_reset_kernel, 1, 1, 0, s, ctrl);
     WalkParams P;
@@ -1272,7 +1273,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
     P.perm = perm;
     P.g_first = g_first;
     P.g_count = g_count;
-    P.g_order = bh_groups_ordered(n, G) ? g_order : nullptr;
+    P.g_order = bh_groups_ordered(set.n, G) ? g_order : nullptr;
     P.rec = nd.rec;
     P.com_m = nd.com_m;
     P.seff = nd.seff;
@@ -1312,7 +1313,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
     }
     // few groups: a block of warps each (same bits), unless the caller sized the grid
     if (blocks_per_sm == 0) {
-        const int rc = launch_walk_team(P, order, G, n, sm_count, s);
+        const int rc = launch_walk_team(P, order, G, set, sm_count, s);
         if (rc <= 0) return rc;
     }
     // one slot per lane: shared memory bounds the blocks per SM, five instead of

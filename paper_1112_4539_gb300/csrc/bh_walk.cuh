@@ -572,7 +572,6 @@ __device__ __forceinline__ int bh_take_particles(int2* q, int& pos, int n, unsig
 
 // A block of warps per group (bh_walk_team.cu), for few enough groups of at most
 // kTeamMaxGroup targets: a BH_* code, or 1 when the set is not for it.
-constexpr int kTeamMaxGroup = 128;
-int launch_walk_team(const WalkParams& P, int order, int G, int n, int sm_count, cudaStream_t s);
+int launch_walk_team(const WalkParams& P, int order, int G, const WalkSet& set, int sm_count, cudaStream_t s);
 
 }  // namespace bh

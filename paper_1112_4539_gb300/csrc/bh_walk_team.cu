@@ -450,38 +450,12 @@ static int bh_team_dispatch(const WalkParams& P, int order, int G, int n, int sm
     }
 }
 
-// Eight warps while every group can have a block of its own at once (two such
-// blocks per SM; the walker, at about 1.5 us per 32 nodes, sets the pace), else
-// four (four blocks per SM, as many walkers again): clumpy 16384, G = 96, 183 us
-// with four and 147 with eight, Plummer 65536, G = 64, 657 and 694.
-// One launch, us, on GB300, groups taken by falling cost on both sides:
-//                                     one warp   block
-//   Plummer 4096, order 1, G = 64          166      75
-//   clumpy 16384, order 2, G = 96          468     125
-//   Plummer 70000, order 1, G = 64         798     470
-//   clumpy 100003, order 2, G = 96         679     540
-//   Plummer 150000, order 2, G = 96       1864    1079
-//   clumpy 150000, order 2, G = 96         830     729
-//   clumpy 200000, order 2, G = 128        904     977
-//   clumpy 100000, order 1, G = 64         283     320
-//   Plummer 120000, order 2, G = 32        505     656
-//   Plummer 262144, order 2, G = 96       1101    1428
-// From about one group per warp of bh_walk_kernel's grid on (16 warps per SM) the
-// groups fill the GPU by themselves and the walkers' idle issue slots cost more
-// than the split gains.  Groups are estimated at 0.65 G particles (measured
-// 0.65-0.75 G).
-static int bh_team_warps(int G, int n, int sm_count)
+// (How many warps a set gets: bh_team_warps in bh_internal.cuh.)
+int launch_walk_team(const WalkParams& P, int order, int G, const WalkSet& set, int sm_count, cudaStream_t s)
 {
-    const double groups = n / (0.65 * G);
-    if (G > kTeamMaxGroup || groups > 16.0 * sm_count) return 0;
-    return groups <= 4.0 * sm_count ? 8 : 4;
-}
-
-int launch_walk_team(const WalkParams& P, int order, int G, int n, int sm_count, cudaStream_t s)
-{
-    switch (bh_team_warps(G, n, sm_count)) {
-        case 8: return bh_team_dispatch<8>(P, order, G, n, sm_count, s);
-        case 4: return bh_team_dispatch<4>(P, order, G, n, sm_count, s);
+    switch (bh_team_warps(set, G, sm_count)) {
+        case 8: return bh_team_dispatch<8>(P, order, G, set.n, sm_count, s);
+        case 4: return bh_team_dispatch<4>(P, order, G, set.n, sm_count, s);
         default: return 1;
     }
 }

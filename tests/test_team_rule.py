@@ -1,0 +1,39 @@
+"""Which sets take the walk with a block of warps per group (bh_team_warps), on a GPU of 152 SMs."""
+import os
+import subprocess
+
+import pytest
+
+SRC = r"""
+#include <cstdio>
+#include "bh_internal.cuh"
+using bh::WalkSet;
+static int batch(int systems, long long each, int G)
+{
+    return bh::bh_team_warps(WalkSet((int)(systems * each), systems, systems * WalkSet::of_system(each, G)), G, 152);
+}
+int main()
+{
+    // single systems: by the particles alone, at most 16 groups per SM
+    for (int n : {1, 4096, 37000, 38000, 151000, 152000}) printf("%d ", bh::bh_team_warps(WalkSet(n, 96), 96, 152));
+    printf("%d %d ", bh::bh_team_warps(WalkSet(1000, 128), 128, 152), bh::bh_team_warps(WalkSet(1000, 129), 129, 152));
+    // a system is a group at least: thousands of small ones, and a few
+    printf("%d %d %d %d ", batch(5000, 5, 96), batch(20000, 4, 64), batch(305, 1, 96), batch(304, 96, 96));
+    // short walks: only while every group has a block at once
+    printf("%d %d %d %d ", batch(256, 256, 64), batch(64, 256, 96), batch(32, 256, 96), batch(2, 512, 96));
+    // long ones: as single systems, of which a batch of one is one
+    printf("%d %d %d %d\n", batch(16, 8192, 96), batch(4, 8192, 96), batch(100, 2048, 64), batch(1, 65536, 96));
+    return 0;
+}
+"""
+
+
+def test_rule(tmp_path):
+    from paper_1112_4539_gb300 import _build as b
+    if not os.path.exists(b.NVCC):
+        pytest.skip("no nvcc")
+    src, exe = tmp_path / "rule.cu", tmp_path / "rule"
+    src.write_text(SRC)
+    subprocess.run([b.NVCC] + b.ARCH + ["-std=c++17", "-I", b.CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+    assert [int(v) for v in out] == [8, 8, 8, 4, 4, 0] + [8, 0] + [0, 0, 0, 8] + [0, 0, 8, 8] + [4, 8, 0, 4]

@@ -309,6 +309,7 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
         bh::launch_init(x->ctrl, s);
     }
     if (N > 0 && !bh::bh_small_set(N, x->deep)) {
+        const bool ordered = bh::bh_groups_ordered(bh::WalkSet(N, x->cfg.group_size));
         bh::launch_bbox(pos, N, x->ctrl, grid_for(x), s);
         bh::launch_keys(pos, N, x->ctrl, x->keys, x->cfg.curve, x->deep, grid_for(x), s);
         bh::launch_sort(x->keys, x->keys_alt, x->vals, x->vals_alt, pos, x->pos_s, N, x->lookback, x->ctrl,
@@ -316,8 +317,8 @@ int tree_build(bh_ctx* x, const float* d_pos_mass, int64_t n, void* stream)
         bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap,
                         x->ctrl, grid_for(x), s);
         bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count,
-                          (int32_t*)x->keys_alt, x->ctrl, grid_for(x), s);
-        x->launches += bh::launches_build(x->deep) - (bh::bh_groups_ordered(N, x->cfg.group_size) ? 1 : 2);
+                          (int32_t*)x->keys_alt, ordered, x->ctrl, grid_for(x), s);
+        x->launches += bh::launches_build(x->deep) - (ordered ? 1 : 2);
     }
     x->launches += 1;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
@@ -761,23 +762,22 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
     const int N = (int)n;
+    const bh::WalkSet set(N, x->batch_filled, x->batch_groups);
     bh::launch_init(x->ctrl, s);
     bh::launch_batch_sort((const float4*)d_pos_mass, x->sys_off, x->nsys, x->keys, x->keys_alt, x->vals, x->vals_alt,
                           x->pos_s, x->sys_of, x->sys_box, x->cfg.curve, x->deep, x->ctrl, s);
     bh::launch_tree(x->keys, x->deep, N, x->cfg.leaf_size, x->dl, x->blk, x->flags, x->nd, x->node_cap, x->ctrl,
                     grid_for(x), s, x->sys_of, x->sys_off);
     bh::launch_groups(x->nd, N, x->cfg.group_size, x->flags, x->blk, x->g_first, x->g_count, (int32_t*)x->keys_alt,
-                      x->ctrl, grid_for(x), s);
+                      bh::bh_groups_ordered(set), x->ctrl, grid_for(x), s);
     bh::launch_moments(x->pos_s, x->keys, x->deep, x->nd, x->cfg.order, theta, x->cfg.fp64_node_threshold,
                        x->cfg.curve, N, x->ctrl, grid_for(x), s, x->sys_of, x->sys_box);
     int rc = bh::launch_walk(x->pos_s, x->vals, x->g_first, x->g_count, (const int32_t*)x->keys_alt, x->nd,
                              x->cfg.order, x->cfg.group_size, eps, (float4*)d_acc_pot, x->ctrl, x->sm_count,
-                             x->cfg.block_threads, x->cfg.blocks_per_sm, bh::WalkSet(N, x->batch_filled, x->batch_groups),
-                             x->deep, s,
-                             nullptr, x->cfg.walk_variant);
+                             x->cfg.block_threads, x->cfg.blocks_per_sm, set, x->deep, s, nullptr, x->cfg.walk_variant);
     if (rc) return rc;
     // init, batch sort, 4 tree, 3 or 4 groups, moments per level, 2 walk
-    x->launches += 2 + 4 + (bh::bh_groups_ordered(N, x->cfg.group_size) ? 4 : 3) +
+    x->launches += 2 + 4 + (bh::bh_groups_ordered(set) ? 4 : 3) +
                    bh::launches_moments(N, x->deep) + bh::kLaunchesForce;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     x->n = n;

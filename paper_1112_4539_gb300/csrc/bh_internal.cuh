@@ -411,9 +411,9 @@ void launch_sort(void* keys, void* keys_alt, uint32_t* vals, uint32_t* vals_alt,
 void launch_tree(const void* keys, bool deep, int n, int n_leaf, uint16_t* dl, uint32_t* blk_lvl, uint8_t* flags,
                  const bh_nodes& nd, int64_t node_cap, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                  const uint32_t* sys = nullptr, const int32_t* sys_off = nullptr);
-// g_order (n words): the groups by falling cost
+// g_order (n words): the groups by falling cost, if `ordered`
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
-                   int32_t* g_count, int32_t* g_order, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);
+                   int32_t* g_count, int32_t* g_order, bool ordered, bh_dev_ctrl* ctrl, int grid, cudaStream_t s);
 void launch_moments(const float4* pos_s, const void* keys, bool deep, const bh_nodes& nd, int order,
                     float theta, int fp64_threshold, int curve, int n, bh_dev_ctrl* ctrl, int grid, cudaStream_t s,
                     const uint32_t* sys = nullptr, const float4* sys_box = nullptr);
@@ -426,9 +426,25 @@ inline bool bh_small_set(int n, bool deep) { return n <= (deep ? 4096 : 8192); }
 bool launch_small_build(const float4* pos, int n, int n_leaf, int G, int curve, bool deep, const bh_nodes& nd,
                         int64_t node_cap, void* keys, uint32_t* vals, float4* pos_s, int32_t* g_first, int32_t* g_count,
                         bh_dev_ctrl* ctrl, cudaStream_t s);
-// Whether the groups of n particles are listed by cost for the walks: not where
-// every group has a block at once (the list costs a launch, 3 us).
-inline bool bh_groups_ordered(int n, int G) { return n > 16384 && n > 200 * G; }
+// What the walks are to expect: the particles, the systems they form (of a
+// batched call) and about how many groups: measured 0.65-0.75 G particles each, a
+// whole system where it is no larger than a group, and one more in every other.
+struct WalkSet {
+    int n, systems = 1;
+    double groups;
+    WalkSet(int n_, int G) : n(n_), groups(n_ / (0.65 * G)) {}
+    WalkSet(int n_, int systems_, double groups_) : n(n_), systems(systems_), groups(groups_) {}
+    static double of_system(long long n, int G) { return n <= 0 ? 0.0 : n <= G ? 1.0 : n / (0.65 * G) + 1.0; }
+    // small systems have short walks (see bh_team_warps)
+    bool short_walks() const { return systems > 1 && n < 2048.0 * systems; }
+};
+// Whether the groups are listed by cost for the walks (a launch, 4 us): not where
+// all of them are walked at once and their order means little, by two blocks per
+// SM or, where walks are short, 16 warps.
+inline bool bh_groups_ordered(const WalkSet& set)
+{
+    return set.n > 16384 && set.groups > (set.short_walks() ? 1600 : 200) / 0.65;
+}
 // One CTA per system: root cube, keys, stable radix sort and gather of each
 // system's particles (systems contiguous, each <= kBatchMaxN particles).
 constexpr int kBatchMaxN = 65536;
@@ -444,17 +460,6 @@ struct WalkLearned {
     const bh_mlp_dev* mlp;
     float theta_guard;
 };
-// What launch_walk is to expect: the particles, the systems they form (of a
-// batched call) and about how many groups: measured 0.65-0.75 G particles each, a
-// whole system where it is no larger than a group, and one more in every other.
-struct WalkSet {
-    int n, systems = 1;
-    double groups;
-    WalkSet(int n_, int G) : n(n_), groups(n_ / (0.65 * G)) {}
-    WalkSet(int n_, int systems_, double groups_) : n(n_), systems(systems_), groups(groups_) {}
-    static double of_system(long long n, int G) { return n <= 0 ? 0.0 : n <= G ? 1.0 : n / (0.65 * G) + 1.0; }
-};
-
 constexpr int kTeamMaxGroup = 128;  // targets per group that the team walk holds
 // Warps per group of the team walk (bh_walk_team.cu), 0: a warp per group
 // (bh_walk_kernel).  Eight while every group can have a block of its own at once
@@ -484,8 +489,7 @@ constexpr int kTeamMaxGroup = 128;  // targets per group that the team walk hold
 // 245 | 234, 16 of 8192 666 | 540, 5000 of 4 to 8 221 | 281.
 inline int bh_team_warps(const WalkSet& set, int G, int sm_count)
 {
-    const bool batch = set.systems > 1 && set.n < 2048.0 * set.systems;
-    if (G > kTeamMaxGroup || set.groups > (batch ? 2.0 : 16.0) * sm_count) return 0;
+    if (G > kTeamMaxGroup || set.groups > (set.short_walks() ? 2.0 : 16.0) * sm_count) return 0;
     return set.groups <= 4.0 * sm_count ? 8 : 4;
 }
 

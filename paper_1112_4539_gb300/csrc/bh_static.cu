@@ -166,6 +166,7 @@ extern "C" int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh
     const int N32 = (int)n;
     const int grid = sd.sm_count * 8;
     const float4* pos = (const float4*)d_pos_mass;
+    const bh::WalkSet set(N32, c.group_size);
     if (bh::bh_small_set(N32, false)) {
         if (!bh::launch_small_build(pos, N32, c.leaf_size, c.group_size, c.curve, false, nd, (int64_t)NN, keys, vals,
                                     pos_s, g_first, g_count, ctrl, s)) {
@@ -181,11 +182,11 @@ extern "C" int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh
         bh::launch_tree(keys, false, N32, c.leaf_size, (uint16_t*)(b + o_dl), (uint32_t*)(b + o_blk),
                         (uint8_t*)(b + o_flags), nd, (int64_t)NN, ctrl, grid, s);
         bh::launch_groups(nd, N32, c.group_size, (uint8_t*)(b + o_flags), (uint32_t*)(b + o_blk), g_first, g_count,
-                          (int32_t*)keys_alt, ctrl, grid, s);
+                          (int32_t*)keys_alt, bh::bh_groups_ordered(set), ctrl, grid, s);
     }
     bh::launch_moments(pos_s, keys, false, nd, c.order, theta, c.fp64_node_threshold, c.curve, N32, ctrl, grid, s);
     int rc = bh::launch_walk(pos_s, vals, g_first, g_count, (const int32_t*)keys_alt, nd, c.order, c.group_size, eps, (float4*)d_acc_pot, ctrl,
-                             sd.sm_count, c.block_threads, c.blocks_per_sm, bh::WalkSet(N32, c.group_size), false, s, nullptr, c.walk_variant);
+                             sd.sm_count, c.block_threads, c.blocks_per_sm, set, false, s, nullptr, c.walk_variant);
     if (rc) return rc;
     if (cudaGetLastError() != cudaSuccess) return BH_ERR_CUDA;
     if (h_status) {

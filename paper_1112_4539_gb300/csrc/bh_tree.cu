@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(256) bh_group_order_kernel(const int32_t* __re
 }
 
 void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* blk, int32_t* g_first,
-                   int32_t* g_count, int32_t* g_order, bh_dev_ctrl* ctrl, int grid, cudaStream_t s)
+                   int32_t* g_count, int32_t* g_order, bool ordered, bh_dev_ctrl* ctrl, int grid, cudaStream_t s)
 {
     if (n <= 0) return;
     const int nblk = (n + kFlagTile - 1) / kFlagTile;
@@ -551,7 +551,7 @@ void launch_groups(const bh_nodes& nd, int n, int G, uint8_t* flags, uint32_t* b
     bh_launch_after(bh_group_mark_kernel, grid, 256, 0, s, nd, G, flags, ctrl);
     bh_launch_after(bh_flag_count_kernel, nblk, kFlagThreads, 0, s, flags, n, blk);
     bh_launch_after(bh_flag_write_kernel, nblk, kFlagThreads, 0, s, flags, n, blk, g_first, g_count, ctrl);
-    if (bh_groups_ordered(n, G))
+    if (ordered)
         bh_launch_after(bh_group_order_kernel, std::min(grid, (n + 255) / 256), 256, 0, s, g_count, g_order, ctrl);
 }
 

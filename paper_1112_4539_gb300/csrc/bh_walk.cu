@@ -1273,7 +1273,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
     P.perm = perm;
     P.g_first = g_first;
     P.g_count = g_count;
-    P.g_order = bh_groups_ordered(set.n, G) ? g_order : nullptr;
+    P.g_order = bh_groups_ordered(set) ? g_order : nullptr;
     P.rec = nd.rec;
     P.com_m = nd.com_m;
     P.seff = nd.seff;

@@ -1,4 +1,5 @@
-"""Which sets take the walk with a block of warps per group (bh_team_warps), on a GPU of 152 SMs."""
+"""Which sets take the walk with a block of warps per group (bh_team_warps), on a GPU of 152 SMs, and which have
+their groups listed by cost (bh_groups_ordered)."""
 import os
 import subprocess
 
@@ -8,10 +9,12 @@ SRC = r"""
 #include <cstdio>
 #include "bh_internal.cuh"
 using bh::WalkSet;
-static int batch(int systems, long long each, int G)
+static WalkSet of(int systems, long long each, int G)
 {
-    return bh::bh_team_warps(WalkSet((int)(systems * each), systems, systems * WalkSet::of_system(each, G)), G, 152);
+    return WalkSet((int)(systems * each), systems, systems * WalkSet::of_system(each, G));
 }
+static int batch(int systems, long long each, int G) { return bh::bh_team_warps(of(systems, each, G), G, 152); }
+static int order(const WalkSet& s) { return bh::bh_groups_ordered(s); }
 int main()
 {
     // single systems: by the particles alone, at most 16 groups per SM
@@ -22,7 +25,10 @@ int main()
     // short walks: only while every group has a block at once
     printf("%d %d %d %d ", batch(256, 256, 64), batch(64, 256, 96), batch(32, 256, 96), batch(2, 512, 96));
     // long ones: as single systems, of which a batch of one is one
-    printf("%d %d %d %d\n", batch(16, 8192, 96), batch(4, 8192, 96), batch(100, 2048, 64), batch(1, 65536, 96));
+    printf("%d %d %d %d ", batch(16, 8192, 96), batch(4, 8192, 96), batch(100, 2048, 64), batch(1, 65536, 96));
+    // by cost: single systems of more than 16384 and 200 G, short walks from 16 groups per SM on
+    printf("%d %d %d %d ", order(WalkSet(16384, 32)), order(WalkSet(16385, 32)), order(WalkSet(19000, 96)), order(WalkSet(19500, 96)));
+    printf("%d %d %d %d\n", order(of(512, 64, 64)), order(of(3000, 64, 64)), order(of(64, 1024, 96)), order(of(16, 8192, 96)));
     return 0;
 }
 """
@@ -36,4 +42,4 @@ def test_rule(tmp_path):
     src.write_text(SRC)
     subprocess.run([b.NVCC] + b.ARCH + ["-std=c++17", "-I", b.CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
-    assert [int(v) for v in out] == [8, 8, 8, 4, 4, 0] + [8, 0] + [0, 0, 0, 8] + [0, 0, 8, 8] + [4, 8, 0, 4]
+    assert [int(v) for v in out] == [8, 8, 8, 4, 4, 0] + [8, 0] + [0, 0, 0, 8] + [0, 0, 8, 8] + [4, 8, 0, 4] + [0, 1, 0, 1] + [0, 1, 0, 1]

@@ -493,6 +493,14 @@ inline int bh_team_warps(const WalkSet& set, int G, int sm_count)
     return set.groups <= 4.0 * sm_count ? 8 : 4;
 }
 
+// Whether the learned walk takes four blocks per SM instead of three: more warps,
+// each slower with fewer registers, pay from about two groups per warp of the
+// three blocks on.  Whole calls, clumpy, order 2, ms, three | four: G = 96 5000
+// 0.301 | 0.359, 50000 0.694 | 0.890, 200000 0.920 | 1.024, 400000 1.537 | 1.520; G = 64
+// 100000 0.616 | 0.743, 200000 0.948 | 0.910; G = 32 50000 0.452 | 0.475, 100000 0.677 |
+// 0.636.  (Above G = 96 both forms take three or fewer.)
+inline bool bh_learned_four(const WalkSet& set, int G, int sm_count) { return G > 96 || set.groups > 24.0 * sm_count; }
+
 int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_first, const int32_t* g_count,
                 const int32_t* g_order,
                 const bh_nodes& nd, int order, int G, float eps, float4* out, bh_dev_ctrl* ctrl,

@@ -38,7 +38,8 @@ namespace bh {
 #endif
 // Learned walk: with the stack of 30-bit keys four blocks fit the shared memory
 // (60.5 KB per block with the deep one), and 128 registers hold it without
-// spills: clumpy 2^22 12.72 -> 12.26 ms against three blocks of 156 registers.
+// spills: clumpy 2^22 12.72 -> 12.26 ms against three blocks of 156 registers (for
+// sets with groups enough, bh_learned_four).
 template <int T, bool LEARNED, int CAP = kStackCap>
 constexpr int bh_walk_min_blocks()
 {
@@ -1290,7 +1291,7 @@ int launch_walk(const float4* pos_s, const uint32_t* perm, const int32_t* g_firs
         P.mfeat = learned->mfeat;
         P.mlp = learned->mlp;
         P.theta_guard = learned->theta_guard;
-        if (!deep)
+        if (!deep && bh_learned_four(set, G, sm_count))
             return bh_walk_dispatch<true, kStackCapFlat>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
         return bh_walk_dispatch<true>(P, order, G, sm_count, block_threads, blocks_per_sm, s);
     }

@@ -1,5 +1,5 @@
-"""Which sets take the walk with a block of warps per group (bh_team_warps), on a GPU of 152 SMs, and which have
-their groups listed by cost (bh_groups_ordered)."""
+"""Which sets take the walk with a block of warps per group (bh_team_warps), on a GPU of 152 SMs, which have their
+groups listed by cost (bh_groups_ordered), and which take the learned walk of four blocks per SM (bh_learned_four)."""
 import os
 import subprocess
 
@@ -29,6 +29,9 @@ int main()
     // by cost: single systems of more than 16384 and 200 G, short walks from 16 groups per SM on
     printf("%d %d %d %d ", order(WalkSet(16384, 32)), order(WalkSet(16385, 32)), order(WalkSet(19000, 96)), order(WalkSet(19500, 96)));
     printf("%d %d %d %d\n", order(of(512, 64, 64)), order(of(3000, 64, 64)), order(of(64, 1024, 96)), order(of(16, 8192, 96)));
+    // 3648 groups
+    printf("%d %d %d %d\n", bh::bh_learned_four(WalkSet(227000, 96), 96, 152), bh::bh_learned_four(WalkSet(228000, 96), 96, 152),
+           bh::bh_learned_four(WalkSet(100000, 32), 32, 152), bh::bh_learned_four(WalkSet(1000, 128), 128, 152));
     return 0;
 }
 """
@@ -42,4 +45,4 @@ def test_rule(tmp_path):
     src.write_text(SRC)
     subprocess.run([b.NVCC] + b.ARCH + ["-std=c++17", "-I", b.CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
-    assert [int(v) for v in out] == [8, 8, 8, 4, 4, 0] + [8, 0] + [0, 0, 0, 8] + [0, 0, 8, 8] + [4, 8, 0, 4] + [0, 1, 0, 1] + [0, 1, 0, 1]
+    assert [int(v) for v in out] == [8, 8, 8, 4, 4, 0] + [8, 0] + [0, 0, 0, 8] + [0, 0, 8, 8] + [4, 8, 0, 4] + [0, 1, 0, 1] + [0, 1, 0, 1] + [0, 1, 1, 1]

@@ -390,10 +390,9 @@ int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh_config* cf
  * will satisfy, of the kind the library's kernels use, so that a deployment
  * can check that such a wait ends and is reported.
  *   which = BH_SELFTEST_TILE_RING: the paired walk's mbarrier wait (gives up
- *           after one second of running time or 2^22 polls, whichever comes
- *           first; while the GPU runs another process, or is stopped in a
- *           debugger, no running time passes but a fiftieth of a second per
- *           stop);
+ *           65536 polls after one second of %globaltimer time has passed, or
+ *           after 2^22 polls: a second during which the GPU ran another process
+ *           does not end a wait);
  *   which = BH_SELFTEST_LOOKBACK:  the sort's decoupled look-back wait
  *           (gives up after 2^22 polls, well under a second);
  *   which = BH_SELFTEST_TMA:       the TMA-staged walk's wait for its bulk

@@ -741,15 +741,15 @@ __device__ __forceinline__ void bh_fence_proxy_async()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 // Wait for this warp's own copies: no early exit on another warp's abort
-// (copies of valid addresses always complete); false after a second of
-// running time (WaitClock) or kWsSpinLimit polls, with BH_ERR_DEVICE_TIMEOUT recorded.
+// (copies of valid addresses always complete); false some polls
+// after a second (WaitLimit) or after kWsSpinLimit polls, with BH_ERR_DEVICE_TIMEOUT recorded.
 __device__ __forceinline__ bool bh_mbar_wait_own(unsigned long long* b, unsigned int parity, bh_dev_ctrl* c)
 {
     if (bh_mbar_try_wait(b, parity)) return true;
-    WaitClock t(bh_globaltimer());
-    for (int i = 0; i < kWsSpinLimit; i++) {
+    WaitLimit lim(bh_globaltimer());
+    for (int i = 0; i < lim.end; i++) {
         if (bh_mbar_try_wait(b, parity)) return true;
-        if ((i & 63) == 63 && t.over(bh_globaltimer())) break;
+        if ((i & 63) == 63) lim.look(i, bh_globaltimer());
     }
     bh_set_error(c, BH_ERR_DEVICE_TIMEOUT);
     return false;

@@ -482,7 +482,7 @@ __device__ __forceinline__ bool bh_mbar_try_wait(unsigned long long* b, unsigned
     return ok != 0u;
 }
 // Wait for the phase of the given parity to complete.  False (with the error
-// recorded) after a second of running time (WaitClock) or after
+// recorded) some polls after a second has passed (WaitLimit) or after
 // kWsSpinLimit polls, whichever comes first; false at once when another warp
 // has aborted.
 __device__ __forceinline__ unsigned long long bh_globaltimer()
@@ -494,12 +494,12 @@ __device__ __forceinline__ unsigned long long bh_globaltimer()
 __device__ __forceinline__ bool bh_mbar_wait(unsigned long long* b, unsigned int parity, bh_dev_ctrl* c)
 {
     if (bh_mbar_try_wait(b, parity)) return true;
-    WaitClock t(bh_globaltimer());
-    for (int i = 0; i < kWsSpinLimit; i++) {
+    WaitLimit lim(bh_globaltimer());
+    for (int i = 0; i < lim.end; i++) {
         if (bh_mbar_try_wait(b, parity)) return true;
         if ((i & 63) == 63) {
             if (*(volatile unsigned int*)&c->abort) return false;
-            if (t.over(bh_globaltimer())) break;
+            lim.look(i, bh_globaltimer());
         }
     }
     bh_set_error(c, BH_ERR_DEVICE_TIMEOUT);

@@ -51,13 +51,13 @@ struct TileSum {
 __device__ __forceinline__ bool bh_turn_wait(const volatile int* turn, int i, bh_dev_ctrl* c)
 {
     if (*turn == i) return true;
-    WaitClock t(bh_globaltimer());
-    for (int k = 0; k < kWsSpinLimit; k++) {
+    WaitLimit lim(bh_globaltimer());
+    for (int k = 0; k < lim.end; k++) {
         if (*turn == i) return true;
         __nanosleep(20);
         if ((k & 63) == 63) {
             if (*(volatile unsigned int*)&c->abort) return false;
-            if (t.over(bh_globaltimer())) break;
+            lim.look(k, bh_globaltimer());
         }
     }
     bh_set_error(c, BH_ERR_DEVICE_TIMEOUT);

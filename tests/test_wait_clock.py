@@ -1,34 +1,35 @@
-"""The time limit of the bounded device waits (csrc/bh_wait.h) on given clock readings."""
+"""The limits of the bounded device waits (csrc/bh_wait.h) on given clock readings."""
 import os
 import subprocess
 
 SRC = r"""
 #include <cstdio>
 #include "bh_wait.h"
-using bh::WaitClock;
-// readings until the wait is over, at most `most`; step(i): nanoseconds between readings i - 1 and i
+// polls of a wait that nothing satisfies, the clock read at every 64th; step(i): nanoseconds since the reading before
 template <class F>
-static long long polls(F step, long long most)
+static long long polls(F step)
 {
     unsigned long long now = 12345678901234ull;
-    WaitClock t(now);
-    for (long long i = 1; i <= most; i++)
-        if (t.over(now += step(i))) return i;
-    return -1;
+    bh::WaitLimit lim(now);
+    long long n = 0;
+    for (int i = 0; i < lim.end; i++, n++)
+        if ((i & 63) == 63) lim.look(i, now += step(i / 64));
+    return n;
 }
 int main()
 {
     const unsigned long long us = 1000ull, ms = 1000 * us, s = 1000 * ms;
-    // one stop of 3 s, or of an hour, and then 900 ms of waiting
-    printf("%d\n", polls([&](long long i) { return i == 5 ? 3 * s : us; }, 900000) == -1);
-    printf("%d\n", polls([&](long long i) { return i == 1 ? 3600 * s : us; }, 900000) == -1);
-    // time slices: off the GPU for 200 ms after each of 30 readings
-    printf("%d\n", polls([&](long long i) { return i % 10 == 0 ? 200 * ms : us; }, 300) == -1);
-    // a wait that nothing satisfies is over after a second
-    const long long n = polls([&](long long) { return 10 * us; }, 10000000);
-    printf("%d\n", n > 99990 && n < 100010);
-    // and, whatever the readings, after a bounded number of long gaps
-    printf("%d\n", polls([&](long long) { return 3600 * s; }, 1000) > 0);
+    const long long more = 65536, most = 1 << 22;
+    // a stop of 3 s, or of an hour, leaves that many polls
+    printf("%d\n", polls([&](int i) { return i == 5 ? 3 * s : us; }) >= more);
+    printf("%d\n", polls([&](int i) { return i == 0 ? 3600 * s : us; }) >= more);
+    // so do time slices, off the GPU for 200 ms after every 640 polls
+    printf("%d\n", polls([&](int i) { return i % 10 == 9 ? 200 * ms : us; }) >= more);
+    // 64 polls take 100 us: over 65536 polls after a second, and at once no more
+    const long long n = polls([&](int) { return 100 * us; });
+    printf("%d\n", n >= 640000 + more && n <= 640000 + more + 130);
+    // no more than 2^22 polls whatever the clock
+    printf("%d\n", polls([&](int) { return us; }) == most && polls([&](int i) { return i == 65535 ? 2 * s : us; }) == most);
     return 0;
 }
 """

@@ -394,7 +394,7 @@ int bh_tree_force_static(const float* d_pos_mass, int64_t n, const bh_config* cf
  *           after 2^22 polls: a second during which the GPU ran another process
  *           does not end a wait);
  *   which = BH_SELFTEST_LOOKBACK:  the sort's decoupled look-back wait
- *           (gives up after 2^22 polls, well under a second);
+ *           (gives up after 2^22 polls, about a second);
  *   which = BH_SELFTEST_TMA:       the TMA-staged walk's wait for its bulk
  *           copies, on an mbarrier told to expect 16 bytes that no copy
  *           delivers (gives up like the tile ring's wait).

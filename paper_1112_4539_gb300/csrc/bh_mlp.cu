@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(256) bh_mlp_batch_grad_kernel(const float* __r
             S.dy[s] = in ? 2.0f * wgt * r / (float)B : 0.f;
         }
         __syncthreads();
-        // back through layer 2 (its derivatives in registers for the thread's 8 units, in memory for all)
+        // back through layer 2 (its derivatives in registers for the thread's units, in memory for all)
         {
             const float dy = S.dy[s];
 #pragma unroll

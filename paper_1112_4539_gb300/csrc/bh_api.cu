@@ -47,7 +47,7 @@ struct bh_ctx {
     // several independent systems
     int nsys = 0;                   // systems of the current layout (0: none)
     int64_t batch_n = 0;            // their total particle count
-    int batch_filled = 0;           // systems with particles
+    int batch_largest = 0;          // particles of the largest
     double batch_groups = 0.0;      // about how many groups they have (bh::WalkSet)
     uint32_t* sys_of = nullptr;     // system of each Morton position
     int32_t* sys_off = nullptr;     // first particle of each system (+ total)
@@ -727,14 +727,14 @@ int bh_batch_layout(bh_ctx* x, const int64_t* h_offsets, int nsys)
     if (nsys > x->cfg.max_systems) return BH_ERR_TOO_LARGE;
     if (h_offsets[0] != 0) return BH_ERR_INVALID;
     std::vector<int32_t> off32((size_t)nsys + 1);
-    int filled = 0;
+    int largest = 0;
     double groups = 0.0;
     for (int s = 0; s < nsys; s++) {
         const int64_t c = h_offsets[s + 1] - h_offsets[s];
         if (c < 0) return BH_ERR_INVALID;
         if (c > bh::kBatchMaxN) return BH_ERR_TOO_LARGE;
         off32[(size_t)s] = (int32_t)h_offsets[s];
-        filled += c > 0;
+        largest = std::max(largest, (int)c);
         groups += bh::WalkSet::of_system(c, x->cfg.group_size);
     }
     if (h_offsets[nsys] > x->max_n) return BH_ERR_TOO_LARGE;
@@ -745,7 +745,7 @@ int bh_batch_layout(bh_ctx* x, const int64_t* h_offsets, int nsys)
         return BH_ERR_CUDA;
     x->nsys = nsys;
     x->batch_n = h_offsets[nsys];
-    x->batch_filled = filled;
+    x->batch_largest = largest;
     x->batch_groups = groups;
     return BH_OK;
 }
@@ -762,7 +762,7 @@ int bh_force_batched(bh_ctx* x, const float* d_pos_mass, float theta, float eps,
     DeviceGuard guard(x->device);
     cudaStream_t s = (cudaStream_t)stream;
     const int N = (int)n;
-    const bh::WalkSet set(N, x->batch_filled, x->batch_groups);
+    const bh::WalkSet set(N, x->batch_largest, x->batch_groups);
     bh::launch_init(x->ctrl, s);
     bh::launch_batch_sort((const float4*)d_pos_mass, x->sys_off, x->nsys, x->keys, x->keys_alt, x->vals, x->vals_alt,
                           x->pos_s, x->sys_of, x->sys_box, x->cfg.curve, x->deep, x->ctrl, s);

@@ -426,24 +426,24 @@ inline bool bh_small_set(int n, bool deep) { return n <= (deep ? 4096 : 8192); }
 bool launch_small_build(const float4* pos, int n, int n_leaf, int G, int curve, bool deep, const bh_nodes& nd,
                         int64_t node_cap, void* keys, uint32_t* vals, float4* pos_s, int32_t* g_first, int32_t* g_count,
                         bh_dev_ctrl* ctrl, cudaStream_t s);
-// What the walks are to expect: the particles, the systems they form (of a
-// batched call) and about how many groups: measured 0.65-0.75 G particles each, a
+// What the walks are to expect: the particles, the largest system of a batched
+// call (0: there is one system) and about how many groups: measured 0.65-0.75 G particles each, a
 // whole system where it is no larger than a group, and one more in every other.
 struct WalkSet {
-    int n, systems = 1;
+    int n, largest = 0;
     double groups;
     WalkSet(int n_, int G) : n(n_), groups(n_ / (0.65 * G)) {}
-    WalkSet(int n_, int systems_, double groups_) : n(n_), systems(systems_), groups(groups_) {}
+    WalkSet(int n_, int largest_, double groups_) : n(n_), largest(largest_), groups(groups_) {}
     static double of_system(long long n, int G) { return n <= 0 ? 0.0 : n <= G ? 1.0 : n / (0.65 * G) + 1.0; }
-    // small systems have short walks (see bh_team_warps)
-    bool short_walks() const { return systems > 1 && n < 2048.0 * systems; }
+    // small systems have short walks (see bh_team_warps); `below`: particles of the largest
+    bool short_walks(int below) const { return largest > 0 && largest < below && largest < n; }
 };
 // Whether the groups are listed by cost for the walks (a launch, 4 us): not where
 // all of them are walked at once and their order means little, by two blocks per
 // SM or, where walks are short, 16 warps.
 inline bool bh_groups_ordered(const WalkSet& set)
 {
-    return set.n > 16384 && set.groups > (set.short_walks() ? 1600 : 200) / 0.65;
+    return set.n > 16384 && set.groups > (set.short_walks(1024) ? 1600 : 200) / 0.65;
 }
 // One CTA per system: root cube, keys, stable radix sort and gather of each
 // system's particles (systems contiguous, each <= kBatchMaxN particles).
@@ -482,14 +482,16 @@ constexpr int kTeamMaxGroup = 128;  // targets per group that the team walk hold
 // groups fill the GPU by themselves and the walkers' idle issue slots cost more
 // than the split gains.  (Near the limit it depends on the set as well: a Plummer
 // sphere, whose walks are long, still gains, clumps or few terms lose up to 13%.)
-// Batched calls of systems of fewer than 2048 particles on average have short walks,
-// for which a block pays only while all groups have one at once.  Whole calls, us,
-// one warp | block, order 1: 256 systems of 256, G = 64 152 | 177, G = 96 155 | 166,
-// 64 of 256, G = 96 120 | 124, 32 of 256 117 | 107, 64 of 2048 303 | 315, 32 of 2048
-// 245 | 234, 16 of 8192 666 | 540, 5000 of 4 to 8 221 | 281.
+// Batched calls whose largest system has fewer than 1024 (2048) particles have short
+// walks, for which a block pays only up to two (eight) groups per SM.  The largest
+// counts, as a batch ends with the walks of its largest system.  Whole calls, us,
+// one warp | block, order 1, G = 96: 64 systems of 256 120 | 124, 32 of 256 117 | 107, 64
+// of 256 to 2000 209 | 188, 128 of 1024 227 | 252, 64 of 1024 191 | 186, 16 of 256 to 4096
+// 264 | 214, 64 of 2048 303 | 315, 16 of 8192 666 | 540, 5000 of 4 to 8 221 | 281.
 inline int bh_team_warps(const WalkSet& set, int G, int sm_count)
 {
-    if (G > kTeamMaxGroup || set.groups > (set.short_walks() ? 2.0 : 16.0) * sm_count) return 0;
+    const double most = set.short_walks(1024) ? 2.0 : set.short_walks(2048) ? 8.0 : 16.0;
+    if (G > kTeamMaxGroup || set.groups > most * sm_count) return 0;
     return set.groups <= 4.0 * sm_count ? 8 : 4;
 }
 

@@ -1003,8 +1003,10 @@ bh_moments_level_kernel(const float4* __restrict__ pos_s, const K* __restrict__ 
 // 1000 monopole 30 -> 20 us, 4096 36 -> 28, clumpy 4096 quadrupole 39 -> 35, 8192
 // 41 -> 38, 16384 45 -> 46; 63-bit keys, 4096, 64 -> 39.  The four levels near the
 // root of any set in one such launch: 100003 71 -> 73 us, 2^24 437 -> 448, not kept.
+// (One block per SM is said to the compiler: left to itself it spills one order's
+// registers, 28.2 us against 28.5 for Plummer 4096, monopole.)
 template <int ORDER, typename K>
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512)
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(512, 1)
 bh_moments_cluster_kernel(const float4* __restrict__ pos_s, const K* __restrict__ keys, bh_nodes nd, float theta,
                           int fp64_threshold, int curve, const bh_dev_ctrl* __restrict__ c,
                           const uint32_t* __restrict__ sys, const float4* __restrict__ sys_box)

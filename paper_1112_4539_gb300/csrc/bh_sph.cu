@@ -209,7 +209,7 @@ __device__ __forceinline__ void bh_sph_tile(const float4* __restrict__ ra, const
 // this is the same on every run, and so are the densities' bits.  The block's
 // warps share the subtrees of about half the search radius: from one level
 // (4) on a dense knot's neighbourhood was a single subtree, of one warp.
-// ms, start of both | 1024 throughout, level 4 | this: clumpy 2^20, 500
+// ms, a warp per group | 1024 throughout, level 4 | this: clumpy 2^20, 500
 // neighbours, G = 32 6.96 | 17.1 | 5.4, 32 neighbours 2.01 | 3.21 | 1.75;
 // uniform 2^20, 500, G = 64 3.80 | 5.29 | 3.05; Plummer 250000, 32, G = 64 10.5 | 2.16 |
 // 2.17.
